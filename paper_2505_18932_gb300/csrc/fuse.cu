@@ -307,10 +307,13 @@ __global__ void __launch_bounds__(256) bounds_overlap_kernel(char *__restrict__ 
 
 template <int KMAX, typename MT, typename T, bool TMP>
 __global__ void __launch_bounds__(32 * FZ_WARPS, GVS_FUSE_MIN_BLOCKS) fuse_kernel(const __grid_constant__ FuseArgs a) {
+    __shared__ int2 tab[(kBoundLevels + 1) * KMAX];
+    fill_slab_table<KMAX>(a, tab, threadIdx.x, 32 * FZ_WARPS);
+    __syncthreads();
     const int nbundles = ((a.Wt + T::bx - 1) / T::bx) * ((a.Ht + T::by - 1) / T::by);
     const int bundle = blockIdx.x * FZ_WARPS + (threadIdx.x >> 5);
     if (bundle >= nbundles) return;  // the whole warp leaves together
-    march_bundle<KMAX, MT, T, TMP>(a, bundle, threadIdx.x & 31);
+    march_bundle<KMAX, MT, T, TMP>(a, tab, bundle, threadIdx.x & 31);
 }
 
 template <int KMAX, typename MT, typename T, bool TMP>

@@ -14,6 +14,10 @@ __global__ void __launch_bounds__(32 * FZ_WARPS, GVS_FUSE_MIN_BLOCKS)
     // each warp keeps its current item's arguments in shared memory (read there by the
     // march, instead of from global memory at every use)
     __shared__ FuseArgs s_args[FZ_WARPS];
+    // the items share the input views and the map layout, so one table serves them all
+    __shared__ int2 tab[(kBoundLevels + 1) * KMAX];
+    fill_slab_table<KMAX>(items[0].args, tab, threadIdx.x, 32 * FZ_WARPS);
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     static_assert(sizeof(FuseArgs) % sizeof(int) == 0, "copied as words");
     // the warp's current item and its bundle range: a warp's bundles come in increasing
@@ -39,7 +43,7 @@ __global__ void __launch_bounds__(32 * FZ_WARPS, GVS_FUSE_MIN_BLOCKS)
             for (int i = lane; i < (int)(sizeof(FuseArgs) / sizeof(int)); i += 32) dst[i] = __ldg(&src[i]);
             __syncwarp();
         }
-        march_bundle<KMAX, MT, T, false, false>(s_args[warp], b - cur_begin, lane);
+        march_bundle<KMAX, MT, T, false, false>(s_args[warp], tab, b - cur_begin, lane);
     }
 }
 
