@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(256) bounds_overlap_kernel(char *__restrict__ 
 }
 
 template <int KMAX, typename MT, typename T, bool TMP>
-__global__ void __launch_bounds__(32 * FZ_WARPS, GVS_FUSE_MIN_BLOCKS) fuse_kernel(const __grid_constant__ FuseArgs a) {
+__global__ void __launch_bounds__(32 * FZ_WARPS, fuse_min_blocks<KMAX, T, TMP>()) fuse_kernel(const __grid_constant__ FuseArgs a) {
     __shared__ int2 tab[(kBoundLevels + 1) * KMAX];
     fill_slab_table<KMAX>(a, tab, threadIdx.x, 32 * FZ_WARPS);
     __syncthreads();

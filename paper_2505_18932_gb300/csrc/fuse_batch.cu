@@ -9,7 +9,7 @@ namespace {
 // taken, and marches it with that item's arguments.  No warp ever waits on
 // another; the counter is reset before each launch.
 template <int KMAX, typename MT, typename T>
-__global__ void __launch_bounds__(32 * FZ_WARPS, GVS_FUSE_MIN_BLOCKS)
+__global__ void __launch_bounds__(32 * FZ_WARPS, fuse_min_blocks<KMAX, T, false>())
     fuse_batch_kernel(const BatchItem *__restrict__ items, int n_items, int total, unsigned *__restrict__ counter) {
     // each warp keeps its current item's arguments in shared memory (read there by the
     // march, instead of from global memory at every use)

@@ -90,10 +90,10 @@ __device__ __forceinline__ void nearest_pixel(float hx, float hy, float hz, int 
 #define GVS_FUSE_WARPS 4        // warps (bundles) per fusion block
 #endif
 constexpr int FZ_WARPS = GVS_FUSE_WARPS;
-#ifndef GVS_FUSE_MIN_BLOCKS
-#define GVS_FUSE_MIN_BLOCKS 9   // resident blocks per SM requested from the register allocator (56 registers)
-#endif
-constexpr int SKIP_COOL = 3;    // samples evaluated after both slab tests fail, before testing again
+// Samples evaluated after both slab tests fail, before testing again: the failing short
+// segment and the sample after it (8 x 1080p, 16 x 1080p with a half2 map: 2: 293 and 570 us,
+// 3: 274 and 557, 4: 293 and 554, at 9 resident blocks).
+constexpr int SKIP_COOL = 3;
 
 // Bundle shape and slab-test lengths of the march.  Every variant computes the
 // same result; they differ only in speed, and the autotuner picks one per
@@ -131,6 +131,19 @@ using Tile4 = Tile<4, 8, 8, 2, false, 2>;
 using Tile5 = Tile<8, 4, 8, 2, false, 2>;
 using Tile6 = Tile<1, 1, 8, 2, false, 1, true>;
 constexpr int kFuseVariants = 7;
+
+// Resident blocks per SM asked of the register allocator, measured over 5 to 12 (us):
+//   8 or 16 views, all of them present: 12 (40 registers; the rays spill to L1 and the warps
+//     hide it): 8 x 1080p 254 against 274 at 9 and 301 at 7; 16 x 1080p, half2 map, 507
+//     against 557 and 621;
+//   up to 4 views: 7 (72 registers), for small targets are one wave of bundles whose time is
+//     one bundle's chain of tests and samples: 4 x 320x240 26.8 against 28.8 at 9;
+//   otherwise (a guard per view, the temporal input, 32 views): 9 (56 registers):
+//     5 views at 961x541 68.0 against 71.7 at 12 and 71.5 at 7.
+template <int KMAX, typename T, bool TMP>
+constexpr int fuse_min_blocks() {
+    return KMAX <= 4 ? 7 : (T::full && !T::warp && !TMP && KMAX <= 16) ? 12 : 9;
+}
 
 struct Ray {
     float ax, ay, az;
@@ -414,14 +427,17 @@ __device__ __forceinline__ void march_rays(const FuseArgs &a, const int2 *tab, i
                 s = min(s + nfree * L, a.D - 1);  // samples up to s are not crossing ends; s is evaluated next
                 if (s == a.D - 1) break;           // ... unless it is the last: nothing follows it
                 have_prev = false;
-                shorter = false;
-                continue;
+                if (nfree == NSEG) {
+                    shorter = false;
+                    continue;
+                }
             }
+            // the segment of length L at s is not free: only shorter ones there can be
             if (!shorter && SKIP_SHORT < SKIP_LONG) {
                 shorter = true;
                 continue;
             }
-            shorter = false;
+            shorter = SKIP_SHORT < SKIP_LONG;  // more often than not the surface is still near
             cool = SKIP_COOL;
         }
         // every lane evaluates (the warp issues the sample anyway); lanes still marching record it
@@ -526,14 +542,16 @@ __device__ __forceinline__ void march_ray_warp(const FuseArgs &a, const int2 *ta
                 s = min(s + nfree * L, a.D - 1);
                 if (s == a.D - 1) break;
                 have_prev = false;
-                shorter = false;
-                continue;
+                if (nfree == NQ) {
+                    shorter = false;
+                    continue;
+                }
             }
             if (!shorter && SKIP_SHORT < SKIP_LONG) {
                 shorter = true;
                 continue;
             }
-            shorter = false;
+            shorter = SKIP_SHORT < SKIP_LONG;  // more often than not the surface is still near
             cool = SKIP_COOL;
         }
         // this lane's term of sample s + tq in view tk, as evaluate_sample forms it
