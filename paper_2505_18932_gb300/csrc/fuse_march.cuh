@@ -214,7 +214,9 @@ __device__ __forceinline__ void fill_slab_table(const FuseArgs &a, int2 *tab, in
 // depth bins (a clear bin holds no depth; see DepthBound), which separates the
 // surfaces of a tile that straddles a depth discontinuity.  When every view is free over the
 // slab, no sample of it can end a crossing (S > 0 wherever W > 0).
-template <int KMAX>
+// AHEAD: free means that no valid depth lies in [zlo - 1.0001 mu, zhi + 1.0001 mu]: every
+// term is not only positive or cut off but saturated (sdf >= 1) or cut off.
+template <int KMAX, bool AHEAD = false>
 __device__ __forceinline__ bool slab_view_free(const FuseArgs &a, const int2 *tab, int k, const SlabRays &r, float z0,
                                                float z1) {
     const float h0lo = __fmaf_rn(z0, r.azlo, r.b2), h0hi = __fmaf_rn(z0, r.azhi, r.b2);
@@ -225,6 +227,7 @@ __device__ __forceinline__ bool slab_view_free(const FuseArgs &a, const int2 *ta
     zlo -= 1e-6f * fabsf(zlo);
     if (zhi <= 1e-6f) return true;  // behind the camera throughout
     if (!front) return false;       // crosses the camera plane: do not try
+    if (AHEAD) zhi = __fadd_ru(zhi, a.behind);
     const float q0hi = fast_rcp(h0lo), q0lo = fast_rcp(h0hi), q1hi = fast_rcp(h1lo), q1lo = fast_rcp(h1hi);
     const auto low = [](float h, float qlo, float qhi) { return h * (h < 0.0f ? qhi : qlo); };
     const auto high = [](float h, float qlo, float qhi) { return h * (h < 0.0f ? qlo : qhi); };
