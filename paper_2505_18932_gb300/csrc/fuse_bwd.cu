@@ -146,173 +146,160 @@ __device__ __forceinline__ int window_multiplicity(int c, int x, int n, int R) {
 }
 
 #ifndef GVS_GATHER_ROWS
-#define GVS_GATHER_ROWS 4  // 8 reads fewer shared values per output but runs fewer warps: 278 -> 312 us
+#define GVS_GATHER_ROWS 4
 #endif
 constexpr int GB_TX = 32;                 // block of 32 x 32 input pixels: 32 x (32 / GB_ROWS) threads,
 constexpr int GB_TY = 32;                 // each thread GB_ROWS consecutive rows
 constexpr int GB_ROWS = GVS_GATHER_ROWS;
 static_assert(GB_TY % GB_ROWS == 0, "the rows split evenly among the thread rows");
 
-// P(c) = A(c) domega/dnu(c) at input pixel (cx, cy) of view k, or 0 outside the
-// image, where A = 0, at an invalid centre (dc NaN) or where the weight is
-// saturated.  dtc: the depth tile at c's window corner (re-sum of nu without a map).
-template <int R, int DW>
-__device__ __forceinline__ float adjoint_p(const float2 *__restrict__ ak, const float2 *__restrict__ wk, int cx,
-                                           int cy, int W, int H, float dc, const float (*dtc)[DW], int ox, float mu,
-                                           float wconst, float inv_w2) {
-    float P = 0.0f;
-    if (cx >= 0 && cx < W && cy >= 0 && cy < H) {
-        const float A = ak[(size_t)cy * W + cx].x;
-        if (A != 0.0f && dc == dc) {
-            if (wk) {
-                const float om = __ldg(&wk[(size_t)cy * W + cx]).y;
-                if (om < 1.0f) P = A * (-0.5f * om * om * om * (inv_w2 / (wconst * wconst)));
-            } else {
-                float nu = 0.0f;
-                for (int dy = 0; dy <= 2 * R; ++dy)
-                    for (int dx = 0; dx <= 2 * R; ++dx) {
-                        const float t = fminf(fabsf(dc - dtc[dy][ox + dx]), mu);
-                        nu = fmaf(t, t, nu);
-                    }
-                const float unclamped = nu > 0.0f ? wconst * rsqrtf(nu * inv_w2) : 2.0f;
-                if (unclamped < 1.0f) P = A * (-0.5f * unclamped / nu);
-            }
-        }
-    }
-    return P;
+// P(c) from A(c) (0 outside the image), the weight omega and the depth d (NaN: invalid).
+__device__ __forceinline__ float adjoint_p(float A, float om, float d, float inv_w2, float wconst) {
+    return (A != 0.0f && d == d && om < 1.0f) ? A * (-0.5f * om * om * om * (inv_w2 / (wconst * wconst))) : 0.0f;
 }
 
-// wmap: the forward's float2 (d, omega) planes, or null (re-sum nu).
-// The P tile holds 2 P(c): every term of the gradient carries the factor 2
-// (d/dd (d - n)^2), and scaling by 2 is exact, so 2 (d_x - d_n)(P(x) + P(n))
-// = (d_x - d_n)(2 P(x) + 2 P(n)) bit for bit with one multiplication fewer per
-// term; the border path halves its own sums instead, again exactly.
-template <int R, typename DT>
+// The same without a stored FP32 weight: nu is summed again from the depth tile dt, whose
+// element [0][ox] is the corner of c's window.
+template <int R, int DW>
+__device__ __forceinline__ float adjoint_p_resum(float A, float d, const float (*dt)[DW], int ox, float mu,
+                                                 float wconst, float inv_w2) {
+    if (!(A != 0.0f && d == d)) return 0.0f;
+    float nu = 0.0f;
+    for (int dy = 0; dy <= 2 * R; ++dy)
+        for (int dx = 0; dx <= 2 * R; ++dx) {
+            const float t = fminf(fabsf(d - dt[dy][ox + dx]), mu);
+            nu = fmaf(t, t, nu);
+        }
+    const float unclamped = nu > 0.0f ? wconst * rsqrtf(nu * inv_w2) : 2.0f;
+    return unclamped < 1.0f ? A * (-0.5f * unclamped / nu) : 0.0f;
+}
+
+// MAP: depths and weights come from the forward's float2 (d, omega) planes; otherwise from
+// `depth`, the weights' nu summed again.
+// The shared tile holds (-d, 2 P) of the outputs and an R halo, depths replicated past the
+// image's borders (NaN: invalid) and P = 0 there.  For a pixel x off the image's edge rows
+// and columns, entry n of its window and the window centre c = n coincide, so its gradient is
+// one pass over the tile: (d_x - d_n) (2 P(x) + 2 P(n)) where |d_x - d_n| < mu (false for an
+// invalid n or x).  The factor 2 of the square's derivative sits in the tile, exactly.  One
+// packed addition gives both factors of a term, the depth test predicates its one FMA, and
+// a thread's GB_ROWS outputs share the values of their window rows.  On an edge
+// row or column the clamped entries of other windows land on x too: those pixels, and
+// only those, add the remaining multiplicity of each window that holds them.  A tile
+// whose P are all 0 (no crossing was sampled there, or every weight is saturated) has
+// grad = B.  8 x 1080p: 278 -> 159 us, 4 x 640x360: 39.7 -> 18.6 us (from separate depth and P
+// tiles, a packed pair's work in two additions, and every block at the border on a
+// scalar path of two windows a pixel).
+template <int R, typename DT, bool MAP>
 __global__ void __launch_bounds__(GB_TX *(GB_TY / GB_ROWS)) fuse_bwd_gather(const DT *__restrict__ depth,
                                                                 const float2 *__restrict__ wmap,
                                                                 const float2 *__restrict__ acc,
                                                                 float *__restrict__ grad, int W, int H, float mu,
                                                                 float wconst, float inv_w2) {
-    constexpr int DW = GB_TX + 4 * R, DH = GB_TY + 4 * R;   // depths: outputs + 2R halo
-    constexpr int PW = GB_TX + 2 * R, PH = GB_TY + 2 * R;   // 2 P(c): outputs + R halo
-    constexpr int TR = GB_TY / GB_ROWS;                     // thread rows
-    static_assert(DW - GB_TX <= GB_TX && PW - GB_TX <= GB_TX, "the halo columns fit one more pass of the lanes");
-    __shared__ float dt[DH][DW];
-    __shared__ float pt[PH][PW];
+    constexpr int DW = GB_TX + 4 * R, DH = GB_TY + 4 * R;   // depths for the re-sum: outputs + 2R halo
+    constexpr int PW = GB_TX + 2 * R, PH = GB_TY + 2 * R;   // (-d, 2 P): outputs + R halo
+    constexpr int THREADS = GB_TX * (GB_TY / GB_ROWS);
+    __shared__ float dt[MAP ? 1 : DH][DW];
+    __shared__ float2 ct[PH][PW];
     const int k = blockIdx.z;
-    const DT *dep = depth + (size_t)k * W * H;
-    const float2 *ak = acc + (size_t)k * W * H;
-    const float2 *wk = wmap ? wmap + (size_t)k * W * H : nullptr;
+    const size_t plane = (size_t)k * W * H;
+    const float2 *ak = acc + plane;
     const int bx = blockIdx.x * GB_TX, by = blockIdx.y * GB_TY;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    {
-        // depth tile by rows: each lane's two clamped columns computed once
-        const int gxa = min(max(bx - 2 * R + tx, 0), W - 1);
-        const int gxb = min(max(bx - 2 * R + GB_TX + tx, 0), W - 1);
-        const bool has_b = tx < DW - GB_TX;
-#pragma unroll 2
-        for (int sy = ty; sy < DH; sy += TR) {
-            const DT *row = dep + (size_t)min(max(by - 2 * R + sy, 0), H - 1) * W;
-            const float da = load_depth(&row[gxa]);
-            dt[sy][tx] = valid_depth(da) ? da : __int_as_float(0x7fc00000);  // NaN marks invalid
-            if (has_b) {
-                const float db = load_depth(&row[gxb]);
-                dt[sy][GB_TX + tx] = valid_depth(db) ? db : __int_as_float(0x7fc00000);
+    const int tid = threadIdx.x;
+    if (!MAP) {
+        for (int e = tid; e < DH * DW; e += THREADS) {
+            const int sy = e / DW, sx = e - sy * DW;
+            const int gx = min(max(bx - 2 * R + sx, 0), W - 1), gy = min(max(by - 2 * R + sy, 0), H - 1);
+            const float d = load_depth(&depth[plane + (size_t)gy * W + gx]);
+            dt[sy][sx] = valid_depth(d) ? d : __int_as_float(0x7fc00000);  // NaN marks invalid
+        }
+        __syncthreads();
+    }
+    bool any = false;
+    constexpr int NL = (PH * PW + THREADS - 1) / THREADS;
+#pragma unroll(MAP ? 3 : 1)
+    for (int n = 0; n < NL; ++n) {
+        const int e = tid + n * THREADS;
+        if (e < PH * PW) {
+            const int py = e / PW, px = e - py * PW;
+            const int cx = bx - R + px, cy = by - R + py;
+            const int gx = min(max(cx, 0), W - 1), gy = min(max(cy, 0), H - 1);
+            const int o = gy * W + gx;
+            const float A = (gx == cx && gy == cy) ? __ldg(&ak[o]).x : 0.0f;
+            float d, P;
+            if (MAP) {
+                const float2 m = __ldg(&wmap[plane + o]);
+                d = m.x > 0.0f ? m.x : __int_as_float(0x7fc00000);
+                P = adjoint_p(A, m.y, d, inv_w2, wconst);
+            } else {
+                d = dt[py + R][px + R];
+                P = adjoint_p_resum<R, DW>(A, d, dt + py, px, mu, wconst, inv_w2);
             }
+            any |= P != 0.0f;
+            ct[py][px] = make_float2(-d, 2.0f * P);
         }
     }
-    __syncthreads();
-    // 2 P(c) on the outputs and an R halo
-#pragma unroll 1
-    for (int py = ty; py < PH; py += TR) {
-        const int cy = by - R + py;
-        pt[py][tx] = 2.0f * adjoint_p<R, DW>(ak, wk, bx - R + tx, cy, W, H, dt[py + R][tx + R], dt + py, tx, mu,
-                                             wconst, inv_w2);
-        if (tx < PW - GB_TX)
-            pt[py][GB_TX + tx] = 2.0f * adjoint_p<R, DW>(ak, wk, bx - R + GB_TX + tx, cy, W, H,
-                                                         dt[py + R][GB_TX + tx + R], dt + py, GB_TX + tx, mu,
-                                                         wconst, inv_w2);
-    }
-    __syncthreads();
-    // a block whose windows of windows stay inside the image sees every window entry once
-    const bool interior = bx >= 2 * R && by >= 2 * R && bx + GB_TX + 2 * R <= W && by + GB_TY + 2 * R <= H;
-    const int x = bx + tx;
-    const int ly0 = ty * GB_ROWS;  // this thread's GB_ROWS consecutive rows
-    if (interior) {
-        // entry n of x's window and window centre c = n coincide: one pass,
-        // (d_x - d_n) (2 P(x) + 2 P(n)) where |d_x - d_n| < mu (false for an invalid n, and
-        // for an invalid x, whose NaN depth fails every test).  The thread's outputs share
-        // their window rows: each shared value is read once and serves every output whose
-        // window holds it, each output taking its entries in the same order as alone.
-        float dx0[GB_ROWS], Px2[GB_ROWS], g[GB_ROWS];
+    const bool work = __syncthreads_or(any);
+    const int lx = tid % GB_TX, x = bx + lx;
+    const int ly0 = (tid / GB_TX) * GB_ROWS;  // this thread's GB_ROWS consecutive rows
+    if (x >= W || by + ly0 >= H) return;
+    float2 own[GB_ROWS];  // (d_x, 2 P(x))
+    float g[GB_ROWS];
+#pragma unroll
+    for (int p = 0; p < GB_ROWS; ++p) g[p] = by + ly0 + p < H ? __ldg(&ak[(size_t)(by + ly0 + p) * W + x]).y : 0.0f;  // B(x)
+    if (work) {
 #pragma unroll
         for (int p = 0; p < GB_ROWS; ++p) {
-            dx0[p] = dt[ly0 + p + 2 * R][tx + 2 * R];
-            Px2[p] = pt[ly0 + p + R][tx + R];
-            g[p] = ak[(size_t)(by + ly0 + p) * W + x].y;  // B(x)
+            const float2 c = ct[ly0 + p + R][lx + R];
+            own[p] = make_float2(-c.x, c.y);
         }
 #pragma unroll
         for (int r = 0; r < GB_ROWS + 2 * R; ++r) {
 #pragma unroll
-            for (int ox = -R; ox <= R; ++ox) {
-                const float dn = dt[ly0 + R + r][tx + 2 * R + ox];
-                const float pn2 = pt[ly0 + r][tx + R + ox];
+            for (int ox = 0; ox <= 2 * R; ++ox) {
+                const float2 c = ct[ly0 + r][lx + ox];
 #pragma unroll
                 for (int p = 0; p < GB_ROWS; ++p) {
-                    if (r - p < 0 || r - p > 2 * R) continue;  // row offset oy = r - p - R outside the window
-                    const float diff = dx0[p] - dn;
-                    if (fabsf(diff) < mu) g[p] = fmaf(diff, Px2[p] + pn2, g[p]);
+                    if (r - p < 0 || r - p > 2 * R) continue;  // a row outside the window
+                    const float2 t = __fadd2_rn(own[p], c);    // (d_x - d_n, 2 P(x) + 2 P(n))
+                    if (fabsf(t.x) < mu) g[p] = fmaf(t.x, t.y, g[p]);
                 }
             }
         }
-#pragma unroll
-        for (int p = 0; p < GB_ROWS; ++p) grad[(size_t)k * W * H + (size_t)(by + ly0 + p) * W + x] = g[p];
-        return;
-    }
+        if (x == 0 || x == W - 1 || by + ly0 == 0 || by + ly0 + GB_ROWS >= H) {
 #pragma unroll 1
-    for (int rr = 0; rr < GB_ROWS; ++rr) {
-        const int ly = ly0 + rr;  // row within the block
-        const int y = by + ly;
-        if (x >= W || y >= H) continue;
-        const float dx0 = dt[ly + 2 * R][tx + 2 * R];
-        float g = ak[(size_t)y * W + x].y;  // B(x)
-        if (dx0 == dx0) {
-            const float Px2 = pt[ly + R][tx + R];
-            if (Px2 != 0.0f) {
-                // P(x) sum 2 (d_x - d_n) = 2 P(x) sum (d_x - d_n): every partial sum halved exactly
-                float sum = 0.0f;
-                for (int ey = -R; ey <= R; ++ey)
-                    for (int ex = -R; ex <= R; ++ex) {
-                        const float dn = dt[ly + 2 * R + ey][tx + 2 * R + ex];
-                        const float diff = dx0 - dn;
-                        if (fabsf(diff) < mu) sum += diff;  // false for a NaN (invalid) neighbour
+            for (int p = 0; p < GB_ROWS; ++p) {
+                const int y = by + ly0 + p;
+                if (y >= H || !(x == 0 || x == W - 1 || y == 0 || y == H - 1)) continue;
+                const float dx = -ct[ly0 + p + R][lx + R].x;
+                float more = 0.0f;
+                for (int oy = -R; oy <= R; ++oy) {
+                    const int my = window_multiplicity(y + oy, y, H, R);
+                    for (int ox = -R; ox <= R; ++ox) {
+                        const int m = my * window_multiplicity(x + ox, x, W, R);
+                        const float2 c = ct[ly0 + p + R + oy][lx + R + ox];
+                        const float diff = dx + c.x;
+                        if (m > 1 && fabsf(diff) < mu) more = fmaf((float)(m - 1) * c.y, diff, more);
                     }
-                g += Px2 * sum;
-            }
-            for (int cyo = -R; cyo <= R; ++cyo) {
-                const int my = window_multiplicity(y + cyo, y, H, R);
-                if (my == 0) continue;
-                for (int cxo = -R; cxo <= R; ++cxo) {
-                    const int mx = window_multiplicity(x + cxo, x, W, R);
-                    if (mx == 0) continue;
-                    const float Pc2 = pt[ly + R + cyo][tx + R + cxo];
-                    if (Pc2 == 0.0f) continue;
-                    const float diff = dt[ly + 2 * R + cyo][tx + 2 * R + cxo] - dx0;
-                    // m P(c) (-2) diff = -(m 2 P(c)) diff
-                    if (fabsf(diff) < mu) g += -((float)(mx * my) * Pc2) * diff;
                 }
+#pragma unroll
+                for (int q = 0; q < GB_ROWS; ++q)
+                    if (q == p) g[q] += more;  // (no dynamic index into registers)
             }
         }
-        grad[(size_t)k * W * H + (size_t)y * W + x] = g;
     }
+#pragma unroll
+    for (int p = 0; p < GB_ROWS; ++p)
+        if (by + ly0 + p < H) grad[plane + (size_t)(by + ly0 + p) * W + x] = g[p];
 }
 
 template <int R, typename DT>
 cudaError_t launch_bwd_gather_r(const void *depth, const float2 *wmap, const float2 *acc, float *grad, int K, int W,
                                 int H, float mu, float wconst, float inv_w2, cudaStream_t st) {
     dim3 grid((W + GB_TX - 1) / GB_TX, (H + GB_TY - 1) / GB_TY, K);
-    fuse_bwd_gather<R, DT><<<grid, dim3(GB_TX, GB_TY / GB_ROWS), 0, st>>>(reinterpret_cast<const DT *>(depth), wmap, acc, grad,
-                                                                W, H, mu, wconst, inv_w2);
+    constexpr int threads = GB_TX * (GB_TY / GB_ROWS);
+    const DT *d = reinterpret_cast<const DT *>(depth);
+    if (wmap) fuse_bwd_gather<R, DT, true><<<grid, threads, 0, st>>>(d, wmap, acc, grad, W, H, mu, wconst, inv_w2);
+    else fuse_bwd_gather<R, DT, false><<<grid, threads, 0, st>>>(d, wmap, acc, grad, W, H, mu, wconst, inv_w2);
     return cudaGetLastError();
 }
 
