@@ -30,14 +30,6 @@ __device__ __forceinline__ void store_map(__half2 *p, float d, float w) { *p = _
 __device__ __forceinline__ float2 load_map(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ float2 load_map(const __half2 *p) { return __half22float2(__ldg(p)); }
 
-// 1 / x for x > 0 within 1 ulp (a denormal x counts as 0), one instruction: the
-// general approximate division adds range scaling around it.
-__device__ __forceinline__ float fast_rcp(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // Nearest integers (ties to even) of the exact real quotients hx/hz, hy/hz,
 // hz > 0.  q = h * r with r = fast_rcp(hz) (1 ulp) and one rounded product is within
 // 3e-7 |q| of the quotient, so n = rint(q) is the answer whenever
@@ -55,17 +47,6 @@ __device__ __forceinline__ float exact_nearest_fixup(float num, float den, float
         else if (lo < 0.0f || (lo == 0.0f && odd)) n -= 1.0f;
     }
     return n;
-}
-
-// Nearest integer by the 1.5 * 2^23 shift: for |q| < 2^22 the sum q + 1.5 * 2^23
-// lies in [2^23, 2^24), where the FP32 values are the integers, so the rounded
-// sum is the shift plus rint(q) (ties to even: the shift is even) and its low
-// bits hold rint(q) + 2^22.  Full-rate additions in place of a round and a
-// conversion.
-__device__ __forceinline__ float shift_round(float q, int &n) {
-    const float t = __fadd_rn(q, 12582912.0f);
-    n = __float_as_int(t) - 0x4B400000;
-    return __fsub_rn(t, 12582912.0f);
 }
 
 // Every |q| >= 2^22 has a margin above 0.5 and takes the exact path; an

@@ -80,6 +80,25 @@ inline MapLayout map_layout(int K, int W, int H) {
 // Depth bin of a value d >= 0 (see DepthBound); the same integer arithmetic in
 // the map build and in the slab test.
 __device__ __forceinline__ int depth_bin(float d) { return (int)(__float_as_uint(d) >> 18); }
+
+// 1 / x for x > 0 within 1 ulp (a denormal x counts as 0), one instruction: the
+// general approximate division adds range scaling around it.
+__device__ __forceinline__ float fast_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Nearest integer by the 1.5 * 2^23 shift: for |q| < 2^22 the sum q + 1.5 * 2^23
+// lies in [2^23, 2^24), where the FP32 values are the integers, so the rounded
+// sum is the shift plus rint(q) (ties to even: the shift is even) and its low
+// bits hold rint(q) + 2^22.  Full-rate additions in place of a round and a
+// conversion.
+__device__ __forceinline__ float shift_round(float q, int &n) {
+    const float t = __fadd_rn(q, 12582912.0f);
+    n = __float_as_int(t) - 0x4B400000;
+    return __fsub_rn(t, 12582912.0f);
+}
 #endif
 
 struct FuseArgs {
@@ -126,7 +145,7 @@ cudaError_t launch_fuse_backward(const FuseArgs &a, const void *depth, int depth
                                  int window, cudaStream_t st);
 
 // ---- forward splat ---------------------------------------------------------
-struct SplatView {
+struct __align__(16) SplatView {  // a view's coefficients in four 16-byte loads
     ViewXform xf;
     float f_ratio;
 };

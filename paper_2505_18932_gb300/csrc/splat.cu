@@ -89,12 +89,12 @@ __device__ __forceinline__ Geo contract(const SplatView &sv, int u, int v, float
 }
 
 // The covered target pixels of the contract above without its correctly
-// rounded divisions.  The three quotients are taken with the fast approximate
-// division (at most 2 ulp from the exact quotient for divisors in
-// [2^-126, 2^126]); each bound is then an integer decision on a value within
+// rounded divisions.  The three quotients are products with one approximate
+// reciprocal (1 ulp, and half an ulp for the product: 1.8e-7 from the exact
+// quotient for divisors in [1e-6, 1e30]); each bound is then an integer decision on a value within
 // eps of the contract's own value.  The worst-case difference of x -/+ hw
-// between the two: 2.5 ulp of the quotient x (2.98e-7 |x|), half of the
-// difference of rho (its quotient 2.5 ulp plus both products' roundings:
+// between the two: 2.98e-7 |x| for the quotient x (it needs 2.4e-7), half of the
+// difference of rho (its quotient 2.4e-7 plus both products' roundings:
 // 4.2e-7 rho, so 4.2e-7 hw after the halving and the clamps) and the two
 // roundings of the sum (1.2e-7 (|x| + hw)): at most 5.4e-7 (|x| + hw); the
 // point mode's nearest pixel needs 3e-7 |x|.  With
@@ -104,15 +104,20 @@ __device__ __forceinline__ Geo contract(const SplatView &sv, int u, int v, float
 // Returns 1 (covered pixels in i0..j1), 0 (no pixel), or -1 when some value is
 // within eps of a boundary or out of the fast division's range: the caller
 // then evaluates the exact contract.  z is h2, computed exactly as there.
-struct Bounds {
-    int i0, i1, j0, j1;
-    float z;
-};
 
-__device__ __forceinline__ float dist_to_integer(float t) { return fabsf(t - rintf(t)); }
+// [ceil(lo), floor(hi)] as integers, |lo|, |hi| < 2^22, from their nearest integers;
+// returns the smaller distance of the two to an integer.
+__device__ __forceinline__ float integers_between(float lo, float hi, int &i0, int &i1) {
+    const float dl = lo - shift_round(lo, i0), dh = hi - shift_round(hi, i1);
+    i0 += dl > 0.0f;
+    i1 -= dh < 0.0f;
+    return fminf(fabsf(dl), fabsf(dh));
+}
 
-__device__ __forceinline__ int contract_bounds_fast(const SplatView &sv, int u, int v, float d, int Wt, int Ht,
-                                                    int footprint, float max_hw, Bounds &o) {
+// One reciprocal serves the three quotients, and full-rate additions give the integer
+// bounds (rounding and conversion instructions run at a fraction of the rate).
+__device__ __forceinline__ int contract_fast(const SplatView &sv, int u, int v, float d, int Wt, int Ht,
+                                             int footprint, float max_hw, Geo &o) {
     if (!valid_depth(d)) return 0;
     const float *A = sv.xf.M;
     const float *c = sv.xf.b;
@@ -125,40 +130,30 @@ __device__ __forceinline__ int contract_bounds_fast(const SplatView &sv, int u, 
     const float h2 = __fmaf_rn(d, m2, c[2]);
     if (!(h2 > 1e-6f)) return 0;
     if (!(h2 < 1e30f)) return -1;
-    const float x = __fdividef(h0, h2);
-    const float y = __fdividef(h1, h2);
-    // far outside any target (|x| < 2^22 keeps eps below one pixel), or NaN: exact path
-    if (!(fabsf(x) < 4.0e6f) || !(fabsf(y) < 4.0e6f)) return -1;
-    float lox, hix, loy, hiy;
+    const float r = fast_rcp(h2);
+    const float x = h0 * r, y = h1 * r;
+    const float hw = footprint ? fminf(fmaxf(0.5f * (sv.f_ratio * (d * r)), 0.5f), max_hw) : 0.0f;
+    const float ax = fabsf(x) + hw, ay = fabsf(y) + hw;
+    // far outside any target (the sums below 2^22 keep eps below a pixel's width and the
+    // nearest integers exact), or NaN: exact path
+    if (!(ax < 4.0e6f) || !(ay < 4.0e6f)) return -1;
+    const float ex = fmaf(1e-6f, ax, 1e-30f), ey = fmaf(1e-6f, ay, 1e-30f);
     if (footprint) {
-        const float rho = __fmul_rn(sv.f_ratio, __fdividef(d, h2));
-        const float hw = fminf(fmaxf(__fmul_rn(0.5f, rho), 0.5f), max_hw);
-        const float a0 = __fsub_rn(x, hw), a1 = __fadd_rn(x, hw);
-        const float b0 = __fsub_rn(y, hw), b1 = __fadd_rn(y, hw);
-        const float ex = 1e-6f * (fabsf(x) + hw) + 1e-30f;
-        const float ey = 1e-6f * (fabsf(y) + hw) + 1e-30f;
-        if (!(fminf(dist_to_integer(a0), dist_to_integer(a1)) > ex) ||
-            !(fminf(dist_to_integer(b0), dist_to_integer(b1)) > ey))
+        if (!(integers_between(x - hw, x + hw, o.i0, o.i1) > ex) ||
+            !(integers_between(y - hw, y + hw, o.j0, o.j1) > ey))
             return -1;
-        lox = ceilf(a0);
-        hix = floorf(a1);
-        loy = ceilf(b0);
-        hiy = floorf(b1);
     } else {
-        const float ex = 1e-6f * fabsf(x) + 1e-30f, ey = 1e-6f * fabsf(y) + 1e-30f;
-        if (!(dist_to_integer(__fsub_rn(x, 0.5f)) > ex) || !(dist_to_integer(__fsub_rn(y, 0.5f)) > ey))
+        // the pixel between x - 1/2 and x + 1/2
+        if (!(integers_between(x - 0.5f, x + 0.5f, o.i0, o.i1) > ex) ||
+            !(integers_between(y - 0.5f, y + 0.5f, o.j0, o.j1) > ey))
             return -1;
-        lox = hix = rintf(x);
-        loy = hiy = rintf(y);
     }
-    if (lox < 0.0f) lox = 0.0f;
-    if (loy < 0.0f) loy = 0.0f;
-    if (hix > (float)(Wt - 1)) hix = (float)(Wt - 1);
-    if (hiy > (float)(Ht - 1)) hiy = (float)(Ht - 1);
-    if (!(lox <= hix) || !(loy <= hiy)) return 0;
-    o.i0 = (int)lox; o.i1 = (int)hix; o.j0 = (int)loy; o.j1 = (int)hiy;
+    o.i0 = max(o.i0, 0);
+    o.j0 = max(o.j0, 0);
+    o.i1 = min(o.i1, Wt - 1);
+    o.j1 = min(o.j1, Ht - 1);
     o.z = h2;
-    return 1;
+    return o.i0 <= o.i1 && o.j0 <= o.j1;
 }
 
 // tag < 32, z > 0 (31 bits), src < 2^28 (GVS_MAX_DIM is 2^14)
@@ -171,32 +166,23 @@ __device__ __forceinline__ float key_depth(unsigned long long key) {
     return __uint_as_float((unsigned)((key >> 28) & 0x7fffffffull));
 }
 
-// Block of 32 x 8 source pixels, grid (ceil(W / 32), ceil(H / 8), views of
-// the group): view, row and column come from the block coordinates, so no
-// integer division.  DT: float or __half depth storage, widened to FP32.
-// REJECT: candidates in front of the fused surface (z < fused - mu_guide)
-// take no part in the depth test.
+// The fast form, or the exact one where it cannot decide; false: no pixel is covered.
+__device__ __forceinline__ bool contract_either(const SplatView &sv, int u, int v, float d, int Wt, int Ht,
+                                                int footprint, float max_hw, Geo &g) {
+    const int ok = contract_fast(sv, u, v, d, Wt, Ht, footprint, max_hw, g);
+    if (ok >= 0) return ok != 0;
+    g = contract(sv, u, v, d, Wt, Ht, footprint, max_hw);
+    return g.ok;
+}
+
+// Blocks of 32 x 8 threads, grid (ceil(W / 32), ceil(H / 8), views of the group): view,
+// row and column come from the block coordinates, so no integer division.
 constexpr int SC_BX = 32, SC_BY = 8;
 
-template <typename DT, bool REJECT = false>
-__global__ void __launch_bounds__(SC_BX * SC_BY) splat_scatter(const SplatArgs a, int k0, unsigned tag) {
-    const int u = blockIdx.x * SC_BX + threadIdx.x;
-    const int v = blockIdx.y * SC_BY + threadIdx.y;
-    if (u >= a.W || v >= a.H) return;
-    const int kk = blockIdx.z;
-    const int k = k0 + kk;
-    const int src = v * a.W + u;
-    const float d = load_depth(reinterpret_cast<const DT *>(a.depth) + (size_t)k * a.W * a.H + src);
-    Bounds b;
-    int ok = contract_bounds_fast(a.v[k], u, v, d, a.Wt, a.Ht, a.footprint, a.max_hw, b);
-    if (ok < 0) {
-        const Geo g = contract(a.v[k], u, v, d, a.Wt, a.Ht, a.footprint, a.max_hw);
-        ok = g.ok;
-        b.i0 = g.i0; b.i1 = g.i1; b.j0 = g.j0; b.j1 = g.j1; b.z = g.z;
-    }
-    if (!ok) return;
-    const unsigned long long key = z_key(tag, b.z, src);
-    unsigned long long *slot = a.keys + (size_t)kk * a.Wt * a.Ht;
+// The key of one source pixel to every target pixel of its footprint.
+template <bool REJECT>
+__device__ __forceinline__ void scatter_pixel(const SplatArgs &a, unsigned long long *slot, const Geo &b,
+                                              unsigned long long key) {
     if (b.j1 - b.j0 <= 1 && b.i1 - b.i0 <= 1) {
         // the usual pixel-sized footprint: at most 2 x 2 pixels, one predicated body
 #pragma unroll
@@ -220,13 +206,45 @@ __global__ void __launch_bounds__(SC_BX * SC_BY) splat_scatter(const SplatArgs a
         }
 }
 
+// SC_ROWS source pixels per thread, SC_BY rows apart (blocks cover 32 x 8 SC_ROWS pixels):
+// their depth loads overlap and the view's coefficients (indexed constants, fetched by a
+// slow unit that was 60 % busy) are fetched once.  8 x 1080p: 112 us with one pixel and the
+// divisions, 107 without them, 89 and 85 with 2 and 4 pixels.
+// DT: float or __half depth storage, widened to FP32.
+// REJECT: candidates in front of the fused surface (z < fused - mu_guide)
+// take no part in the depth test.
+constexpr int SC_ROWS = 4;
+template <typename DT, bool REJECT = false>
+__global__ void __launch_bounds__(SC_BX * SC_BY) splat_scatter(const SplatArgs a, int k0, unsigned tag) {
+    const int u = blockIdx.x * SC_BX + threadIdx.x;
+    const int v0 = blockIdx.y * (SC_BY * SC_ROWS) + threadIdx.y;
+    if (u >= a.W) return;
+    const int kk = blockIdx.z;
+    const int k = k0 + kk;
+    const DT *depth = reinterpret_cast<const DT *>(a.depth) + (size_t)k * a.W * a.H;
+    unsigned long long *slot = a.keys + (size_t)kk * a.Wt * a.Ht;
+    float d[SC_ROWS];
+#pragma unroll
+    for (int n = 0; n < SC_ROWS; ++n) {
+        const int v = v0 + n * SC_BY;
+        d[n] = v < a.H ? load_depth(depth + v * a.W + u) : 0.0f;  // 0: no pixel
+    }
+#pragma unroll
+    for (int n = 0; n < SC_ROWS; ++n) {
+        const int v = v0 + n * SC_BY;
+        Geo b;
+        if (contract_either(a.v[k], u, v, d[n], a.Wt, a.Ht, a.footprint, a.max_hw, b))
+            scatter_pixel<REJECT>(a, slot, b, z_key(tag, b.z, v * a.W + u));
+    }
+}
+
 // 31 for the first group of views of a call, then falling (at most 32 groups of >= 1 view)
 inline unsigned group_tag(int group) { return 31u - (unsigned)group; }
 static_assert(GVS_MAX_VIEWS <= 32, "a group's tag has 5 bits");
 static_assert((int64_t)GVS_MAX_DIM * GVS_MAX_DIM <= (int64_t)1 << 28, "a source index has 28 bits");
 
-inline dim3 scatter_grid(int W, int H, int kn) {
-    return dim3((unsigned)((W + SC_BX - 1) / SC_BX), (unsigned)((H + SC_BY - 1) / SC_BY), (unsigned)kn);
+inline dim3 scatter_grid(int W, int H, int kn, int rows = 1) {
+    return dim3((unsigned)((W + SC_BX - 1) / SC_BX), (unsigned)((H + SC_BY * rows - 1) / (SC_BY * rows)), (unsigned)kn);
 }
 
 // has: some candidate of this group (tag) reached the pixel; then w is the winner's source
@@ -847,7 +865,7 @@ void soft_groups(const SplatArgs &a, int K, cudaStream_t st) {
         const int kn = (K - k0) < slots ? (K - k0) : slots;
         const unsigned tag = group_tag(k0 / slots);
         const bool reset = k0 + kn < K;  // the accumulators serve another group
-        splat_scatter<DT><<<scatter_grid(a.W, a.H, kn), dim3(SC_BX, SC_BY), 0, st>>>(a, k0, tag);
+        splat_scatter<DT><<<scatter_grid(a.W, a.H, kn, SC_ROWS), dim3(SC_BX, SC_BY), 0, st>>>(a, k0, tag);
         soft_accum<DT, CT><<<scatter_grid(a.W, a.H, kn), dim3(SC_BX, SC_BY), 0, st>>>(a, k0);
         if (tma_soft_resolve_ok(a, HWt))
             soft_resolve_tma<<<dim3((unsigned)((HWt + ST_PX - 1) / ST_PX), (unsigned)kn), 256, 0, st>>>(a, k0, tag, reset);
@@ -876,7 +894,7 @@ cudaError_t launch_splat(const SplatArgs &a, int K, cudaStream_t st) {
     }
     for (int k0 = 0; k0 < K; k0 += slots) {
         const int kn = (K - k0) < slots ? (K - k0) : slots;
-        const dim3 g = scatter_grid(a.W, a.H, kn), b(SC_BX, SC_BY);
+        const dim3 g = scatter_grid(a.W, a.H, kn, SC_ROWS), b(SC_BX, SC_BY);
         const unsigned tag = group_tag(k0 / slots);
         if (a.depth_dtype == GVS_F16) {
             if (a.guide_reject) splat_scatter<__half, true><<<g, b, 0, st>>>(a, k0, tag);
