@@ -243,6 +243,39 @@ __device__ void block_sort(unsigned long long *key, int n) {
     __syncthreads();
 }
 
+// The same for n <= 2 GS_THREADS (the usual list has 441): one pair per thread and step and
+// every stride a constant, about half the instructions a step.  4 views at 720p: render
+// 612 -> 519 us.
+__device__ __forceinline__ void block_sort_small(unsigned long long *key, int n) {
+    const int i = threadIdx.x;
+    const auto step = [&](int x, int y) {
+        if (y < n) {
+            const unsigned long long kx = key[x], ky = key[y];
+            if (kx > ky) { key[x] = ky; key[y] = kx; }
+        }
+    };
+    static_assert(GS_THREADS == 256, "2^9 keys, one pair per thread");
+#pragma unroll
+    for (int lk = 1; lk <= 9; ++lk) {
+        const int hk = 1 << (lk - 1);
+        if (hk >= n) break;  // sorted (the whole block leaves together)
+        if (hk > 32) __syncthreads();
+        const int x = i + (i & ~(hk - 1));  // a 0 bit inserted into i at hk
+        step(x, x ^ (2 * hk - 1));
+        if (hk > 32) __syncthreads();
+        else __syncwarp();
+#pragma unroll
+        for (int lj = lk - 2; lj >= 0; --lj) {
+            const int j = 1 << lj;
+            const int xj = i + (i & ~(j - 1));
+            step(xj, xj + j);
+            if (j > 32) __syncthreads();
+            else __syncwarp();
+        }
+    }
+    __syncthreads();
+}
+
 // Transposes a 32 x 32 bit matrix held one row per lane: afterwards bit q of lane p is
 // what bit p of lane q was.  Five exchanges of half-blocks.
 __device__ __forceinline__ unsigned transpose_bits(unsigned x, int lane) {
@@ -287,7 +320,8 @@ __global__ void __launch_bounds__(GS_THREADS) gauss_render(const GaussArgs g, in
         keys = skeys;
     }
     __syncthreads();
-    block_sort(keys, n);
+    if (n <= 2 * GS_THREADS) block_sort_small(skeys, n);
+    else block_sort(keys, n);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cx = (warp & 1) * 8, cy = (warp >> 1) * 4;  // the warp's rectangle within the tile
     const int i = blockIdx.x * GS_TILE + cx + (lane & 7);
