@@ -29,71 +29,24 @@ namespace {
 // so they are bit-identical to it.
 // ---------------------------------------------------------------------------
 
-// One target pixel with a crossing: recompute its two bracketing samples and
-// add each contributing view's terms at the sampled input pixel.
-template <int KMAX, typename MT, bool FULL>
-__device__ __forceinline__ void bwd_pixel(const FuseArgs &a, int i, int j, int s, float G, float2 *__restrict__ acc) {
-    const float fi = (float)i, fj = (float)j;
-    Ray ray[KMAX];
-#pragma unroll
-    for (int k = 0; k < KMAX; ++k) {
-        if (FULL || k < a.K) {
-            const float *M = a.xf[k].M;
-            ray[k].ax = __fmaf_rn(M[0], fi, __fmaf_rn(M[1], fj, M[2]));
-            ray[k].ay = __fmaf_rn(M[3], fi, __fmaf_rn(M[4], fj, M[5]));
-            ray[k].az = __fmaf_rn(M[6], fi, __fmaf_rn(M[7], fj, M[8]));
-        }
-    }
-    const float z0 = __fmaf_rn((float)s, a.dz, a.zn), z1 = __fmaf_rn((float)(s + 1), a.dz, a.zn);
-    float S0, S1, W0, W1;
-    evaluate_sample<KMAX, MT, FULL>(a, ray, z0, S0, W0);
-    evaluate_sample<KMAX, MT, FULL>(a, ray, z1, S1, W1);
-    const float den = (S0 - S1) * (S0 - S1);
-    const float gS[2] = {G * (z1 - z0) * (-S1) / den, G * (z1 - z0) * S0 / den};
-    const MT *map = reinterpret_cast<const MT *>(a.dw);
-    const size_t plane = (size_t)a.W * a.H;
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const float zs = t ? z1 : z0;
-#pragma unroll
-        for (int k = 0; k < KMAX; ++k) {
-            if (FULL || k < a.K) {
-                const float hz = __fmaf_rn(zs, ray[k].az, a.xf[k].b[2]);
-                if (hz > 1e-6f) {
-                    const float hx = __fmaf_rn(zs, ray[k].ax, a.xf[k].b[0]);
-                    const float hy = __fmaf_rn(zs, ray[k].ay, a.xf[k].b[1]);
-                    int u, v;
-                    nearest_pixel(hx, hy, hz, u, v);
-                    if ((unsigned)u < (unsigned)a.W && (unsigned)v < (unsigned)a.H) {
-                        const size_t q = (size_t)k * plane + (size_t)v * a.W + u;
-                        const float2 p = load_map(&map[q]);
-                        const float sdf = (p.x - hz) * a.inv_mu;
-                        if (sdf >= -1.0f && p.y > 0.0f) {
-                            const float c = fminf(sdf, 1.0f);
-                            const float inband = (sdf > -1.0f && sdf < 1.0f) ? a.inv_mu : 0.0f;
-                            atomicAdd(&acc[q], make_float2(gS[t] * c, gS[t] * p.y * inband));
-                        }
-                    }
-                }
-            }
-        }
-    }
-}
-
 // Pass 1.  Only target pixels with a crossing (and a non-zero upstream
 // gradient) have work, about a third of them on the 8 x 1080p frame; so each
 // block of 128 threads first lists the pixels with work among its 16 x 32 tile
 // (in raster order, through a block-wide prefix count of warp ballots) and then
-// deals the list out to its threads, which keeps the warps full.  Its gathers
-// and atomics wait on memory: twelve resident blocks per SM (40 registers, a few
-// spilled) hide more of that than eight at 64 registers (130.8 -> 123.3 us).
-// FULL: the call has exactly KMAX views (no per-view guard).
-constexpr int BS_TX = 16, BS_TY = 32, BS_THREADS = 128;
-template <int KMAX, typename MT, bool FULL>
-__global__ void __launch_bounds__(BS_THREADS, 12) fuse_bwd_scatter(const FuseArgs a, const int16_t *__restrict__ crossing,
-                                                               const float *__restrict__ grad_fused,
-                                                               float2 *__restrict__ acc) {
+// deals the list out, a group of KMAX lanes to a pixel and a lane to a view: the lane
+// keeps its view's coefficients, gathers the map at both samples, adds the
+// group's terms to S_s and S_{s+1} in view order (the forward's own order and
+// operations, so the same bits) and, with its terms still in registers, issues its two
+// atomics.  8 x 1080p: 121 -> 107 us against a thread to a pixel, which recomputed every
+// term after the sums; resident blocks 8 (64 registers), 12, 16: 107, 115, 112 us.
+constexpr int BS_TX = 16, BS_TY = 32, BS_THREADS = 128, BS_BLOCKS = 8;
+template <int KMAX, typename MT>
+__global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const __grid_constant__ FuseArgs a,
+                                                                         const int16_t *__restrict__ crossing,
+                                                                         const float *__restrict__ grad_fused,
+                                                                         float2 *__restrict__ acc) {
     constexpr int PER = BS_TX * BS_TY / BS_THREADS;  // pixels per thread in the listing pass
+    constexpr int GROUPS = BS_THREADS / KMAX;        // pixels at a time
     __shared__ int s_list[BS_TX * BS_TY];
     __shared__ int s_warp[BS_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -119,11 +72,56 @@ __global__ void __launch_bounds__(BS_THREADS, 12) fuse_bwd_scatter(const FuseArg
         __syncthreads();  // s_warp is rewritten by the next round
         base = total;
     }
-    for (int q = tid; q < base; q += BS_THREADS) {
-        const int e = s_list[q];
+    const int k = tid % KMAX, first = lane - lane % KMAX;  // this lane's view; its group's first lane
+    const ViewXform xf = a.xf[k < a.K ? k : 0];
+    const size_t plane = (size_t)a.W * a.H;
+    const MT *map = reinterpret_cast<const MT *>(a.dw) + (k < a.K ? (size_t)k * plane : 0);
+    float2 *acc_k = acc + (k < a.K ? (size_t)k * plane : 0);
+    for (int q0 = warp * (32 / KMAX); q0 < base; q0 += GROUPS) {  // the same for the whole warp
+        const int q = q0 + lane / KMAX;
+        const bool on = q < base;
+        const int e = s_list[on ? q : q0];
         const int i = blockIdx.x * BS_TX + (e % BS_TX), j = blockIdx.y * BS_TY + (e / BS_TX);
         const size_t o = (size_t)j * a.Wt + i;
-        bwd_pixel<KMAX, MT, FULL>(a, i, j, crossing[o], grad_fused[o], acc);
+        const int s = crossing[o];
+        const float G = grad_fused[o];
+        const float fi = (float)i, fj = (float)j;
+        const float ax = __fmaf_rn(xf.M[0], fi, __fmaf_rn(xf.M[1], fj, xf.M[2]));
+        const float ay = __fmaf_rn(xf.M[3], fi, __fmaf_rn(xf.M[4], fj, xf.M[5]));
+        const float az = __fmaf_rn(xf.M[6], fi, __fmaf_rn(xf.M[7], fj, xf.M[8]));
+        float zs[2], w[2], c[2], inband[2];
+        int at[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            zs[t] = __fmaf_rn((float)(s + t), a.dz, a.zn);
+            const float hz = __fmaf_rn(zs[t], az, xf.b[2]);
+            const float hx = __fmaf_rn(zs[t], ax, xf.b[0]);
+            const float hy = __fmaf_rn(zs[t], ay, xf.b[1]);
+            int u, v;
+            nearest_pixel(hx, hy, hz, u, v);
+            const bool in = k < a.K && hz > 1e-6f && (unsigned)u < (unsigned)a.W && (unsigned)v < (unsigned)a.H &&
+                            GVS_IN_BOUNDS((size_t)k * plane + (size_t)v * a.W + u, (size_t)a.K * plane,
+                                          GVS_SITE_FUSE_MAP);
+            at[t] = in ? v * a.W + u : 0;
+            float2 p = make_float2(0.0f, 0.0f);
+            if (in) p = load_map(map + at[t]);
+            const float sdf = (p.x - hz) * a.inv_mu;
+            w[t] = (in && sdf >= -1.0f) ? p.y : 0.0f;
+            c[t] = w[t] != 0.0f ? fminf(sdf, 1.0f) : 0.0f;
+            inband[t] = (sdf > -1.0f && sdf < 1.0f) ? a.inv_mu : 0.0f;
+        }
+        float S0 = 0.0f, S1 = 0.0f;
+#pragma unroll
+        for (int g = 0; g < KMAX; ++g) {
+            S0 = fmaf(__shfl_sync(0xffffffffu, w[0], first + g), __shfl_sync(0xffffffffu, c[0], first + g), S0);
+            S1 = fmaf(__shfl_sync(0xffffffffu, w[1], first + g), __shfl_sync(0xffffffffu, c[1], first + g), S1);
+        }
+        const float den = (S0 - S1) * (S0 - S1);
+        const float gS[2] = {G * (zs[1] - zs[0]) * (-S1) / den, G * (zs[1] - zs[0]) * S0 / den};
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+            if (on && w[t] > 0.0f)
+                atomicAdd(&acc_k[at[t]], make_float2(gS[t] * c[t], gS[t] * w[t] * inband[t]));
     }
 }
 
@@ -131,8 +129,7 @@ template <int KMAX, typename MT>
 void bwd_scatter_k(const FuseArgs &a, const int16_t *crossing, const float *grad_fused, float2 *acc,
                    cudaStream_t st) {
     const dim3 grid((a.Wt + BS_TX - 1) / BS_TX, (a.Ht + BS_TY - 1) / BS_TY), block(BS_THREADS);
-    if (a.K == KMAX) fuse_bwd_scatter<KMAX, MT, true><<<grid, block, 0, st>>>(a, crossing, grad_fused, acc);
-    else fuse_bwd_scatter<KMAX, MT, false><<<grid, block, 0, st>>>(a, crossing, grad_fused, acc);
+    fuse_bwd_scatter<KMAX, MT><<<grid, block, 0, st>>>(a, crossing, grad_fused, acc);
 }
 
 // Entries e in [-R, R] of a clamp-to-edge window centred at c that land on x
