@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 import torch
@@ -193,8 +194,30 @@ def take_device_status() -> int:
     return int(load().gvs_take_device_status())
 
 
+# gvs_camera in one call; field by field takes several times as long, and a training step
+# hands over 20 cameras
+_CAMERA = struct.Struct("=2i16d")
+assert _CAMERA.size == ctypes.sizeof(GvsCamera)
+
+
+def _camera_bytes(c) -> bytes:
+    """gvs_camera from any object with width, height, fx, fy, cx, cy, R (3x3), t (3)."""
+    try:
+        R, t = c.R, c.t
+        r0, r1, r2 = R.tolist() if hasattr(R, "tolist") else R
+        (a, b, d), (e, f, g), (h, i, j) = r0, r1, r2
+        x, y, z = t.tolist() if hasattr(t, "tolist") else t
+        return _CAMERA.pack(int(c.width), int(c.height), c.fx, c.fy, c.cx, c.cy, a, b, d, e, f, g, h, i, j, x, y, z)
+    except (TypeError, ValueError, struct.error):
+        return bytes(_camera_by_field(c))  # other forms of R (nine values), strings and the like
+
+
 def camera_struct(c) -> GvsCamera:
     """gvs_camera from any object with width, height, fx, fy, cx, cy, R (3x3), t (3)."""
+    return GvsCamera.from_buffer_copy(_camera_bytes(c))
+
+
+def _camera_by_field(c) -> GvsCamera:
     s = GvsCamera()
     s.width, s.height = int(c.width), int(c.height)
     s.fx, s.fy, s.cx, s.cy = float(c.fx), float(c.fy), float(c.cx), float(c.cy)
@@ -209,10 +232,9 @@ def camera_struct(c) -> GvsCamera:
 
 
 def camera_array(cams):
-    arr = (GvsCamera * max(1, len(cams)))()
-    for k, c in enumerate(cams):
-        arr[k] = camera_struct(c)
-    return arr
+    if len(cams) == 0:
+        return (GvsCamera * 1)()
+    return (GvsCamera * len(cams)).from_buffer_copy(b"".join([_camera_bytes(c) for c in cams]))
 
 
 def _ptr(t):
@@ -226,8 +248,10 @@ def _ptr(t):
 
 
 def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    # torch.cuda.current_stream().cuda_stream without building the Stream object
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def depth_dtype_of(t) -> int:
@@ -408,12 +432,15 @@ class FuseDepth(torch.autograd.Function):
         ctx.save_for_backward(in_depths, ws, crossing)
         ctx.cams, ctx.target, ctx.cfg = in_cams, target, cfg
         ctx.mark_non_differentiable(crossing)
+        ctx.set_materialize_grads(False)  # no zeros are made for the crossing's gradient
         return fused, crossing
 
     @staticmethod
     def backward(ctx, grad_fused, grad_crossing):
         in_depths, ws, crossing = ctx.saved_tensors
         cfg = ctx.cfg
+        if grad_fused is None:
+            grad_fused = torch.zeros(crossing.shape, dtype=torch.float32, device=crossing.device)
         g = fuse_depth_backward(ctx.cams, in_depths, ctx.target, cfg["num_samples"], cfg["z_near"], cfg["z_far"],
                                 cfg["mu"], ws, crossing, grad_fused, weight_const=cfg.get("weight_const", 0.001),
                                 window=cfg.get("window", 7))
@@ -790,6 +817,7 @@ class SoftSplat(torch.autograd.Function):
         ctx.save_for_backward(in_depths, in_color, fwd["winner"], fwd["color"], fwd["depth"], fwd["wsum"])
         ctx.cams, ctx.target, ctx.cfg = in_cams, target, cfg
         ctx.mark_non_differentiable(fwd["alpha"])
+        ctx.set_materialize_grads(False)  # an output without a gradient (alpha; often the depth) adds nothing
         return fwd["color"], fwd["depth"], fwd["alpha"]
 
     @staticmethod
