@@ -41,9 +41,10 @@ class BatchPlan:
         self.cross = [[torch.empty((t.height, t.width), dtype=torch.int16, device=dev) for t in self.targets]
                       for _ in range(self.F)]
         big = max(t.width * t.height for t in self.targets)
-        # room for two z-buffers of the largest target (two views per splat pass; smaller
-        # targets fit more), which stays L2-resident next to the streamed outputs
-        self.ws_splat = gvs.workspace(2 * gvs.splat_workspace_bytes(N, big, 1), dev)
+        # z-buffers for at least two views of the largest target, and as many as stay L2-resident
+        # next to the streamed outputs (smaller targets fit more views per splat pass)
+        one = gvs.splat_workspace_bytes(N, big, 1)
+        self.ws_splat = gvs.workspace(max(2 * one, min(N * one, gvs.SPLAT_L2_BYTES)), dev)
         self.splat = [[{k: torch.empty((N, t.height, t.width), dtype=dt, device=dev)
                         for k, dt in (("winner", torch.int32), ("warped_rgba", torch.int32),
                                       ("warped_depth", torch.float32), ("alpha", torch.uint8),
