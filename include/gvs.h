@@ -369,11 +369,11 @@ GVS_API gvs_status gvs_soft_splat_backward(const gvs_camera *in_cams, const void
  * Batched fusion: many (frame, target) items in one persistent launch (a serving
  * pattern; the paper has no counterpart, each item is Supplement A.1's fusion).  Each
  * item fuses the map of one frame (gvs_weight_map) into one target camera,
- * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  The
- * launch keeps every SM busy with one grid that takes bundles of target pixels
- * from a global counter until all items are done (no block waits on another),
- * and is a plain kernel launch plus a 4-byte reset, so it can be captured in a
- * CUDA graph.
+ * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  A target
+ * of about a device-wide wave or more takes a launch of its own; the others share
+ * one grid that keeps every SM busy, taking bundles of target pixels from a global
+ * counter until all of them are done (no block waits on another).  These are plain
+ * kernel launches plus a 4-byte reset, so they can be captured in a CUDA graph.
  */
 typedef struct {
     const void *map;           /* the frame's map, as from gvs_weight_map */

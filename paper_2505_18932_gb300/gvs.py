@@ -844,6 +844,10 @@ class SoftSplat(torch.autograd.Function):
         return gd, gc.to(in_color.dtype), None, None, None
 
 
+# Target pixels from which the library gives an item of a batch a launch of its own.
+FUSE_BATCH_OWN_LAUNCH = 200000
+
+
 class FuseBatch:
     """Batched fusion of many (map, target) items in one persistent launch (gvs_fuse_batch_*).
 
