@@ -93,6 +93,8 @@ void launch_typed(const uint32_t *rgba_t, const uint32_t *rgba_prev, const void 
 // upsample and blend.  Quarter grids live in the workspace.  Each pass runs on
 // blocks of 32 x 8 cells or pixels with the view in blockIdx.z (no index division).
 // ---------------------------------------------------------------------------
+// V4: a cell's four pixels of a row in one 16-byte load (W a multiple of 4, planes aligned).
+template <bool V4>
 __global__ void __launch_bounds__(256) soft_quarter(const uint32_t *__restrict__ rgba_t,
                                                     const uint32_t *__restrict__ rgba_prev, float *__restrict__ mq,
                                                     int W, int H, int Wq, int Hq, int K, float inv_lambda,
@@ -103,14 +105,33 @@ __global__ void __launch_bounds__(256) soft_quarter(const uint32_t *__restrict__
     const size_t off = (size_t)k * W * H;
     float sum = 0.0f;
     int cnt = 0;
-    for (int y = 4 * qy; y < min(4 * qy + 4, H); ++y)
-        for (int x = 4 * qx; x < min(4 * qx + 4, W); ++x) {
-            const size_t p = off + (size_t)y * W + x;
-            const uint32_t d = __vabsdiffu4(__ldg(&rgba_t[p]), __ldg(&rgba_prev[p]));
-            const uint32_t m = max(max(d & 0xffu, (d >> 8) & 0xffu), (d >> 16) & 0xffu);
-            sum += (float)m;
-            ++cnt;
+    const auto largest = [](uint32_t a, uint32_t b) {
+        const uint32_t d = __vabsdiffu4(a, b);
+        return (float)max(max(d & 0xffu, (d >> 8) & 0xffu), (d >> 16) & 0xffu);
+    };
+    if (V4) {
+        uint4 a[4], b[4];
+        cnt = 4 * min(4, H - 4 * qy);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const size_t p = off + (size_t)min(4 * qy + r, H - 1) * W + 4 * qx;
+            a[r] = __ldg(reinterpret_cast<const uint4 *>(rgba_t + p));
+            b[r] = __ldg(reinterpret_cast<const uint4 *>(rgba_prev + p));
         }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (4 * qy + r < H)  // sums of integers below 2^24: exact in any order
+                sum += (largest(a[r].x, b[r].x) + largest(a[r].y, b[r].y)) +
+                       (largest(a[r].z, b[r].z) + largest(a[r].w, b[r].w));
+        }
+    } else {
+        for (int y = 4 * qy; y < min(4 * qy + 4, H); ++y)
+            for (int x = 4 * qx; x < min(4 * qx + 4, W); ++x) {
+                const size_t p = off + (size_t)y * W + x;
+                sum += largest(__ldg(&rgba_t[p]), __ldg(&rgba_prev[p]));
+                ++cnt;
+            }
+    }
     const float mean = sum / (255.0f * (float)cnt);
     mq[q] = fminf(fmaf(mean, inv_lambda, beta), 1.0f);
 }
@@ -136,12 +157,33 @@ __device__ __forceinline__ void st_depth(float *p, float v) { *p = v; }
 __device__ __forceinline__ void st_depth(__half *p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ bool valid_d(float d) { return isfinite(d) && d > 0.0f; }
 
+// Four depths as they are stored, moved by one 16- or 8-byte access.
+__device__ __forceinline__ void ld4(const float *p, float (&v)[4]) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void ld4(const __half *p, float (&v)[4]) {
+    const uint2 t = *reinterpret_cast<const uint2 *>(p);
+    const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&t.x));
+    const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&t.y));
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void st4(float *p, const float (&v)[4]) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st4(__half *p, const float (&v)[4]) {
+    const __half2 a = __floats2half2_rn(v[0], v[1]), b = __floats2half2_rn(v[2], v[3]);
+    *reinterpret_cast<uint2 *>(p) = make_uint2(*reinterpret_cast<const unsigned *>(&a), *reinterpret_cast<const unsigned *>(&b));
+}
+
 // SB_V consecutive pixels of a row per thread: they share the row's vertical
 // interpolation terms and keep more loads in flight; each pixel's arithmetic is
-// the single-pixel form, in the same order.
+// the single-pixel form, in the same order.  V4: every plane moves in vectors of the
+// four pixels (W a multiple of 4, planes aligned); single accesses 16 bytes apart cost four
+// partial sectors each: 8 x 720p 34 us.
 constexpr int SB_V = 4;
 
-template <typename T>
+template <typename T, bool V4>
 __global__ void __launch_bounds__(256) soft_blend(const float *__restrict__ pq, const T *__restrict__ depth_t,
                                                   T *__restrict__ state, float *__restrict__ mask, int W, int H,
                                                   int Wq, int Hq, int K) {
@@ -154,23 +196,39 @@ __global__ void __launch_bounds__(256) soft_blend(const float *__restrict__ pq, 
     const float fy = sy - (float)y0;
     const float *m0 = m + y0 * Wq, *m1 = m + y1 * Wq;
     const size_t row = ((size_t)k * H + y) * W;
+    float dn[SB_V], dp[SB_V], mv[SB_V];
+    if (V4) {
+        ld4(depth_t + row + xs, dn);
+        ld4(state + row + xs, dp);
+    } else {
+#pragma unroll
+        for (int e = 0; e < SB_V; ++e) {
+            dn[e] = xs + e < W ? ld_depth(&depth_t[row + xs + e]) : 0.0f;
+            dp[e] = xs + e < W ? ld_depth(&state[row + xs + e]) : 0.0f;
+        }
+    }
 #pragma unroll
     for (int e = 0; e < SB_V; ++e) {
         const int x = xs + e;
-        if (x >= W) break;
-        const size_t p = row + x;
         const float sx = fminf(fmaxf((x + 0.5f) * 0.25f - 0.5f, 0.0f), (float)(Wq - 1));
         const int x0 = (int)sx;
         const int x1 = min(x0 + 1, Wq - 1);
         const float fx = sx - (float)x0;
         const float M = (1.0f - fy) * ((1.0f - fx) * m0[x0] + fx * m0[x1]) + fy * ((1.0f - fx) * m1[x0] + fx * m1[x1]);
-        if (mask) mask[p] = M;
-        const float dn = ld_depth(&depth_t[p]), dp = ld_depth(&state[p]);
-        float out;
-        if (!valid_d(dp)) out = dn;
-        else if (!valid_d(dn)) out = dp;
-        else out = fmaf(M, dn - dp, dp);  // M dn + (1 - M) dp
-        st_depth(&state[p], out);
+        mv[e] = M;
+        if (!valid_d(dp[e])) dp[e] = dn[e];
+        else if (valid_d(dn[e])) dp[e] = fmaf(M, dn[e] - dp[e], dp[e]);  // M dn + (1 - M) dp
+    }
+    if (V4) {
+        if (mask) st4(mask + row + xs, mv);
+        st4(state + row + xs, dp);
+    } else {
+#pragma unroll
+        for (int e = 0; e < SB_V; ++e) {
+            if (xs + e >= W) break;
+            if (mask) mask[row + xs + e] = mv[e];
+            st_depth(&state[row + xs + e], dp[e]);
+        }
     }
 }
 
@@ -183,10 +241,18 @@ cudaError_t launch_soft_typed(const uint32_t *rgba_t, const uint32_t *rgba_prev,
     float *mq = ws, *pq = ws + nq;
     (void)n;
     const dim3 block(32, 8), gq((Wq + 31) / 32, (Hq + 7) / 8, K), gp((W + 32 * SB_V - 1) / (32 * SB_V), (H + 7) / 8, K);
-    soft_quarter<<<gq, block, 0, st>>>(rgba_t, rgba_prev, mq, W, H, Wq, Hq, K, 1.0f / lambda_t, beta);
+    const auto aligned = [](const void *q, size_t a) { return (uintptr_t)q % a == 0; };
+    if (W % 4 == 0 && aligned(rgba_t, 16) && aligned(rgba_prev, 16))
+        soft_quarter<true><<<gq, block, 0, st>>>(rgba_t, rgba_prev, mq, W, H, Wq, Hq, K, 1.0f / lambda_t, beta);
+    else
+        soft_quarter<false><<<gq, block, 0, st>>>(rgba_t, rgba_prev, mq, W, H, Wq, Hq, K, 1.0f / lambda_t, beta);
     soft_pool<<<gq, block, 0, st>>>(mq, pq, Wq, Hq, K);
-    soft_blend<T><<<gp, block, 0, st>>>(pq, reinterpret_cast<const T *>(depth_t), reinterpret_cast<T *>(state), mask,
-                                        W, H, Wq, Hq, K);
+    const T *d = reinterpret_cast<const T *>(depth_t);
+    T *s = reinterpret_cast<T *>(state);
+    if (W % SB_V == 0 && aligned(d, 4 * sizeof(T)) && aligned(s, 4 * sizeof(T)) && aligned(mask, 16))
+        soft_blend<T, true><<<gp, block, 0, st>>>(pq, d, s, mask, W, H, Wq, Hq, K);
+    else
+        soft_blend<T, false><<<gp, block, 0, st>>>(pq, d, s, mask, W, H, Wq, Hq, K);
     return cudaGetLastError();
 }
 
