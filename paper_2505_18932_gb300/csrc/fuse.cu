@@ -28,6 +28,13 @@ constexpr int WM_TX = 32;   // block of 32 x 64 output pixels: 32 x 8 threads,
 constexpr int WM_P = 8;     // each thread a column of WM_P pixels (8: 3 % faster than 4 at 1080p)
 constexpr int WM_TY = 8 * WM_P;
 
+// x << n, 0 for n > 31
+__device__ __forceinline__ unsigned shl_sat(unsigned x, unsigned n) {
+    unsigned r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+
 // R = window / 2.  The shared tile holds the block's depths, as the map will
 // store them, plus an R-pixel halo replicated at the image borders (invalid
 // depths as NaN).  A thread reads each of the (WM_P + 2R) x (2R + 1) shared
@@ -37,7 +44,8 @@ constexpr int WM_TY = 8 * WM_P;
 // operations (bit-reproducible on the host, as the sphere-tracing path needs);
 // otherwise with the approximate reciprocal square root.
 // 8 resident blocks per SM (32 registers): the stencil needs the warps more
-// than the registers (at 51 registers 10 % slower).
+// than the registers (at 51 registers 10 % slower).  8 x 1080p: 122 -> 119 us since the
+// epilogue tests nothing per pixel where a warp's pixels are all valid.
 template <int R, typename DT, typename MT, bool EXACT = false>
 __global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict__ depth, char *__restrict__ map,
                                                          MapLayout L, float mu, float wconst, float inv_w2) {
@@ -85,13 +93,10 @@ __global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict
     // add and one packed FMA: |dc - n| = |n + (-dc)| exactly, and each output
     // still sums its taps in the same order with the same roundings.
     static_assert(WM_P % 2 == 0, "outputs are paired");
-    float dc[WM_P];
-    float2 ndc[WM_P / 2], nu[WM_P / 2];
-#pragma unroll
-    for (int p = 0; p < WM_P; ++p) dc[p] = tile[ty * WM_P + p + R][tx + R].x;
+    float2 ndc[WM_P / 2], nu[WM_P / 2];  // -dc and nu of each pair
 #pragma unroll
     for (int q = 0; q < WM_P / 2; ++q) {
-        ndc[q] = make_float2(-dc[2 * q], -dc[2 * q + 1]);
+        ndc[q] = make_float2(-tile[ty * WM_P + 2 * q + R][tx + R].x, -tile[ty * WM_P + 2 * q + 1 + R][tx + R].x);
         nu[q] = make_float2(0.0f, 0.0f);
     }
 #pragma unroll
@@ -120,25 +125,34 @@ __global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict
             }
         }
     }
+    float nd[WM_P];  // -dc, NaN where there is no valid pixel
+#pragma unroll
+    for (int p = 0; p < WM_P; ++p) nd[p] = (p & 1) ? ndc[p >> 1].y : ndc[p >> 1].x;
+    const bool inside = x < W && yb + WM_P <= H;
+    if (!inside) {
+#pragma unroll
+        for (int p = 0; p < WM_P; ++p)
+            if (x >= W || yb + p >= H) nd[p] = __int_as_float(0x7fc00000);
+    }
+    // every pixel of the warp valid (the sum of its depths is not NaN): no test per pixel below
+    float sum = nd[0];
+#pragma unroll
+    for (int p = 1; p < WM_P; ++p) sum += nd[p];
+    const bool all_valid = __all_sync(0xffffffffu, sum == sum);
     float lo = kInf, hi = -kInf;
-    MT *dw = reinterpret_cast<MT *>(map + L.off_dw) + (size_t)k * W * H;
+    MT *dw = reinterpret_cast<MT *>(map + L.off_dw) + (size_t)k * W * H + (size_t)yb * W + x;
 #pragma unroll
     for (int p = 0; p < WM_P; ++p) {
-        const int y = yb + p;
-        if (x < W && y < H) {
-            float d = 0.0f, w = 0.0f;
-            if (dc[p] == dc[p]) {  // valid centre
-                const float n = (p & 1) ? nu[p >> 1].y : nu[p >> 1].x;
-                if (EXACT)
-                    w = n > 0.0f ? fminf(__fdiv_rn(wconst, __fsqrt_rn(__fmul_rn(n, inv_w2))), 1.0f) : 1.0f;
-                else
-                    w = n > 0.0f ? fminf(wconst * rsqrtf(n * inv_w2), 1.0f) : 1.0f;
-                d = dc[p];
-                lo = fminf(lo, d);
-                hi = fmaxf(hi, d);
-            }
-            store_map(&dw[(size_t)y * W + x], d, w);
-        }
+        const float n = (p & 1) ? nu[p >> 1].y : nu[p >> 1].x;
+        // n = 0 gives infinity (NaN for wconst = 0), so 1; lo and hi pass a NaN by
+        float d = -nd[p];
+        float w = EXACT ? fminf(__fdiv_rn(wconst, __fsqrt_rn(__fmul_rn(n, inv_w2))), 1.0f)
+                        : fminf(wconst * rsqrtf(n * inv_w2), 1.0f);
+        lo = fminf(lo, d);
+        hi = fmaxf(hi, d);
+        if (!all_valid && !(d == d)) d = w = 0.0f;
+        if (inside || (x < W && yb + p < H)) store_map(dw, d, w);
+        dw += W;
     }
     // 16x16 tile bounds: over the 16 lanes of a tile's columns, then its two thread rows
     static_assert(WM_P == 8 && WM_TX % 16 == 0 && WM_TY % 16 == 0, "a 16x16 tile is 16 lanes x 2 thread rows");
@@ -151,13 +165,27 @@ __global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict
     __syncthreads();
     const float tlo = fminf(red[ty & ~1][tx >> 4].x, red[ty | 1][tx >> 4].x);
     const float thi = fmaxf(red[ty & ~1][tx >> 4].y, red[ty | 1][tx >> 4].y);
-    // the tile's mask: the bin of every valid depth in it, relative to the bin of the smallest
-    unsigned long long mask = 0;
+    // the tile's mask: the bin of every valid depth in it, relative to the bin of the smallest.
+    // shl_sat(1, b) is 0 for b of 32 or more, as for the negative b - 32 of a low bin.
+    unsigned mlo = 0u, mhi = 0u;
     const int base = depth_bin(tlo);
+    if (all_valid) {
 #pragma unroll
-    for (int p = 0; p < WM_P; ++p)
-        if (x < W && yb + p < H && dc[p] == dc[p]) mask |= 1ull << min(depth_bin(dc[p]) - base, kDepthBins - 1);
-    unsigned mlo = (unsigned)mask, mhi = (unsigned)(mask >> 32);
+        for (int p = 0; p < WM_P; ++p) {
+            const int b = min(depth_bin(-nd[p]) - base, kDepthBins - 1);
+            mlo |= shl_sat(1u, (unsigned)b);
+            mhi |= shl_sat(1u, (unsigned)(b - 32));
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < WM_P; ++p) {
+            const int b = min(depth_bin(-nd[p]) - base, kDepthBins - 1);
+            if (nd[p] == nd[p]) {
+                mlo |= shl_sat(1u, (unsigned)b);
+                mhi |= shl_sat(1u, (unsigned)(b - 32));
+            }
+        }
+    }
 #pragma unroll
     for (int m = 1; m < 16; m <<= 1) {
         mlo |= __shfl_xor_sync(0xffffffffu, mlo, m);
