@@ -46,8 +46,10 @@ __device__ __forceinline__ unsigned shl_sat(unsigned x, unsigned n) {
 // 8 resident blocks per SM (32 registers): the stencil needs the warps more
 // than the registers (at 51 registers 10 % slower).  8 x 1080p: 122 -> 119 us since the
 // epilogue tests nothing per pixel where a warp's pixels are all valid.
+// Windows above 9 x 9 get 64 registers: at 32 they spill hundreds of bytes, and the 15 x 15
+// kernel then summed wrong terms for the first output of each thread.
 template <int R, typename DT, typename MT, bool EXACT = false>
-__global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict__ depth, char *__restrict__ map,
+__global__ void __launch_bounds__(256, R <= 4 ? 8 : 4) weight_map_kernel(const DT *__restrict__ depth, char *__restrict__ map,
                                                          MapLayout L, float mu, float wconst, float inv_w2) {
     constexpr int SW = WM_TX + 2 * R;
     constexpr int SH = WM_TY + 2 * R;

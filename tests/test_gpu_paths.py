@@ -48,7 +48,7 @@ def test_gauss_list_lengths(gvs, oracle_mod, target):
     gauss_case(gvs, oracle_mod, w, target=t)
 
 
-@pytest.mark.parametrize("size,window", [((12, 9), 9), ((32, 32), 7), ((33, 34), 7), ((65, 31), 5), ((38, 70), 9)])
+@pytest.mark.parametrize("size,window", [((12, 9), 15), ((40, 30), 15), ((12, 9), 9), ((32, 32), 7), ((33, 34), 7), ((65, 31), 5), ((38, 70), 9)])
 def test_grad_at_borders(gvs, oracle_mod, size, window):
     from synth import configs
     w = configs.tiny(*size, 3, 96)
