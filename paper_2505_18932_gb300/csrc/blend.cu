@@ -22,77 +22,128 @@ __device__ __forceinline__ bool valid_depth(float d) { return isfinite(d) && d >
 __device__ __forceinline__ void store(float *p, float v) { *p = v; }
 __device__ __forceinline__ void store(__half *p, float v) { *p = __float2half_rn(v); }
 __device__ __forceinline__ void store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void store_v(float *p, const float (&v)[2]) { *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]); }
+__device__ __forceinline__ void store_v(__half *p, const float (&v)[2]) {
+    *reinterpret_cast<__half2 *>(p) = __floats2half2_rn(v[0], v[1]);
+}
+__device__ __forceinline__ void store_v(__nv_bfloat16 *p, const float (&v)[2]) {
+    *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(v[0], v[1]);
+}
+template <typename T>
+__device__ __forceinline__ void store_v(T *p, const float (&v)[1]) { store(p, v[0]); }
 __device__ __forceinline__ float load(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+__device__ __forceinline__ void load_v(const float *p, float (&v)[1]) { v[0] = __ldg(p); }
+__device__ __forceinline__ void load_v(const float *p, float (&v)[2]) {
+    const float2 t = __ldg(reinterpret_cast<const float2 *>(p));
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void load_v(const uint32_t *p, uint32_t (&v)[1]) { v[0] = __ldg(p); }
+__device__ __forceinline__ void load_v(const uint32_t *p, uint32_t (&v)[2]) {
+    const uint2 t = __ldg(reinterpret_cast<const uint2 *>(p));
+    v[0] = t.x; v[1] = t.y;
+}
+__device__ __forceinline__ void load_v(const uint8_t *p, float (&v)[1]) { v[0] = (float)__ldg(p); }
+__device__ __forceinline__ void load_v(const uint8_t *p, float (&v)[2]) {
+    const uchar2 t = __ldg(reinterpret_cast<const uchar2 *>(p));
+    v[0] = (float)t.x; v[1] = (float)t.y;
+}
+__device__ __forceinline__ float channel(uint32_t c, int n) { return (float)((c >> (8 * n)) & 0xffu) * (1.0f / 255.0f); }
 
-template <typename OT>
+inline bool aligned_to(const void *p, uintptr_t a) { return ((uintptr_t)p % a) == 0; }
+
+// The normal of the fused depth at (i, j) (0 where a neighbour is missing), D valid there.
+__device__ __forceinline__ void normal_at(const BlendArgs &a, int i, int j, float D, float &n0, float &n1, float &n2) {
+    n0 = n1 = n2 = 0.0f;
+    if (!(i > 0 && i < a.Wt - 1 && j > 0 && j < a.Ht - 1)) return;
+    const size_t p = (size_t)j * a.Wt + i;
+    const float dl = __ldg(&a.fused[p - 1]), dr = __ldg(&a.fused[p + 1]);
+    const float du = __ldg(&a.fused[p - a.Wt]), dd = __ldg(&a.fused[p + a.Wt]);
+    if (!(valid_depth(dl) && valid_depth(dr) && valid_depth(du) && valid_depth(dd))) return;
+    // central differences of the back-projected points, written without
+    // subtracting two large coordinates
+    const float fi = (float)i - a.cx, fj = (float)j - a.cy;
+    const float dh = dr - dl, sh = dr + dl, dv = dd - du, sv = dd + du;
+    const float a0 = (dh * fi + sh) / a.fx, a1 = dh * fj / a.fy, a2 = dh;
+    const float b0 = dv * fi / a.fx, b1 = (dv * fj + sv) / a.fy, b2 = dv;
+    n0 = a1 * b2 - a2 * b1;
+    n1 = a2 * b0 - a0 * b2;
+    n2 = a0 * b1 - a1 * b0;
+    const float P0 = D * fi / a.fx, P1 = D * fj / a.fy;
+    if (n0 * P0 + n1 * P1 + n2 * D > 0.0f) {
+        n0 = -n0;
+        n1 = -n1;
+        n2 = -n2;
+    }
+    const float l2 = n0 * n0 + n1 * n1 + n2 * n2;
+    if (l2 > 0.0f) {
+        const float inv = rsqrtf(l2);
+        n0 *= inv;
+        n1 *= inv;
+        n2 *= inv;
+    }
+}
+
+// V neighbouring pixels per thread (2: even width, arrays aligned to pairs), so that a warp
+// stores 128 bytes of a 16-bit plane at once instead of 64.
+// 4 views at 1352x1014 in bfloat16: 40 -> 33 us.
+template <typename OT, int V>
 __global__ void __launch_bounds__(256) features_kernel(const BlendArgs a, OT *__restrict__ out) {
-    const int i = blockIdx.x * 32 + threadIdx.x;
+    const int i = (blockIdx.x * 32 + threadIdx.x) * V;
     const int j = blockIdx.y * 8 + threadIdx.y;
     if (i >= a.Wt || j >= a.Ht) return;
     const int K = a.K;
     const size_t np = (size_t)a.Wt * a.Ht;
     const size_t p = (size_t)j * a.Wt + i;
+    float D[V], n[V][3], P[V][3], rl[V];
+    bool have[V];
+    load_v(a.fused + p, D);
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        have[e] = valid_depth(D[e]);
+        n[e][0] = n[e][1] = n[e][2] = P[e][0] = P[e][1] = P[e][2] = rl[e] = 0.0f;
+        if (have[e]) {
+            normal_at(a, i + e, j, D[e], n[e][0], n[e][1], n[e][2]);
+            P[e][0] = D[e] * ((float)(i + e) - a.cx) / a.fx;
+            P[e][1] = D[e] * ((float)j - a.cy) / a.fy;
+            P[e][2] = D[e];
+            rl[e] = rsqrtf(P[e][0] * P[e][0] + P[e][1] * P[e][1] + P[e][2] * P[e][2]);
+        }
+    }
+    store_v(out + (size_t)(5 * K) * np + p, D);
     for (int k = 0; k < K; ++k) {
         const size_t o = (size_t)k * np + p;
-        const uint32_t c = __ldg(&a.rgba[o]);
-        store(&out[(size_t)(3 * k + 0) * np + p], (float)(c & 0xffu) * (1.0f / 255.0f));
-        store(&out[(size_t)(3 * k + 1) * np + p], (float)((c >> 8) & 0xffu) * (1.0f / 255.0f));
-        store(&out[(size_t)(3 * k + 2) * np + p], (float)((c >> 16) & 0xffu) * (1.0f / 255.0f));
-        store(&out[(size_t)(3 * K + k) * np + p], __ldg(&a.wdepth[o]));
-        store(&out[(size_t)(4 * K + k) * np + p], (float)__ldg(&a.alpha[o]));
-        store(&out[(size_t)(7 * K + 1 + k) * np + p], a.dist[k]);
-        store(&out[(size_t)(8 * K + 1 + k) * np + p], a.axis[k]);
-    }
-    const float D = __ldg(&a.fused[p]);
-    store(&out[(size_t)(5 * K) * np + p], D);
-    const bool have = valid_depth(D);
-    float n0 = 0.0f, n1 = 0.0f, n2 = 0.0f;
-    if (have && i > 0 && i < a.Wt - 1 && j > 0 && j < a.Ht - 1) {
-        const float dl = __ldg(&a.fused[p - 1]), dr = __ldg(&a.fused[p + 1]);
-        const float du = __ldg(&a.fused[p - a.Wt]), dd = __ldg(&a.fused[p + a.Wt]);
-        if (valid_depth(dl) && valid_depth(dr) && valid_depth(du) && valid_depth(dd)) {
-            // central differences of the back-projected points, written without
-            // subtracting two large coordinates
-            const float fi = (float)i - a.cx, fj = (float)j - a.cy;
-            const float dh = dr - dl, sh = dr + dl, dv = dd - du, sv = dd + du;
-            const float a0 = (dh * fi + sh) / a.fx, a1 = dh * fj / a.fy, a2 = dh;
-            const float b0 = dv * fi / a.fx, b1 = (dv * fj + sv) / a.fy, b2 = dv;
-            n0 = a1 * b2 - a2 * b1;
-            n1 = a2 * b0 - a0 * b2;
-            n2 = a0 * b1 - a1 * b0;
-            const float P0 = D * fi / a.fx, P1 = D * fj / a.fy;
-            if (n0 * P0 + n1 * P1 + n2 * D > 0.0f) {
-                n0 = -n0;
-                n1 = -n1;
-                n2 = -n2;
-            }
-            const float l2 = n0 * n0 + n1 * n1 + n2 * n2;
-            if (l2 > 0.0f) {
-                const float inv = rsqrtf(l2);
-                n0 *= inv;
-                n1 *= inv;
-                n2 *= inv;
+        uint32_t c[V];
+        float wd[V], al[V], v[V], nd[V], rd[V];
+        load_v(a.rgba + o, c);
+        load_v(a.wdepth + o, wd);
+        load_v(a.alpha + o, al);
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) v[e] = channel(c[e], ch);
+            store_v(out + (size_t)(3 * k + ch) * np + p, v);
+        }
+        store_v(out + (size_t)(3 * K + k) * np + p, wd);
+        store_v(out + (size_t)(4 * K + k) * np + p, al);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            nd[e] = rd[e] = 0.0f;
+            if (have[e]) {
+                const float d0 = P[e][0] - a.ck[k][0], d1 = P[e][1] - a.ck[k][1], d2 = P[e][2] - a.ck[k][2];
+                const float il = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+                nd[e] = (n[e][0] * d0 + n[e][1] * d1 + n[e][2] * d2) * il;
+                rd[e] = (P[e][0] * d0 + P[e][1] * d1 + P[e][2] * d2) * il * rl[e];
             }
         }
-    }
-    float P0 = 0.0f, P1 = 0.0f, P2 = 0.0f, rl = 0.0f;
-    if (have) {
-        P0 = D * ((float)i - a.cx) / a.fx;
-        P1 = D * ((float)j - a.cy) / a.fy;
-        P2 = D;
-        rl = rsqrtf(P0 * P0 + P1 * P1 + P2 * P2);
-    }
-    for (int k = 0; k < K; ++k) {
-        float nd = 0.0f, rd = 0.0f;
-        if (have) {
-            const float d0 = P0 - a.ck[k][0], d1 = P1 - a.ck[k][1], d2 = P2 - a.ck[k][2];
-            const float il = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
-            nd = (n0 * d0 + n1 * d1 + n2 * d2) * il;
-            rd = (P0 * d0 + P1 * d1 + P2 * d2) * il * rl;
-        }
-        store(&out[(size_t)(5 * K + 1 + k) * np + p], nd);
-        store(&out[(size_t)(6 * K + 1 + k) * np + p], rd);
+        store_v(out + (size_t)(5 * K + 1 + k) * np + p, nd);
+        store_v(out + (size_t)(6 * K + 1 + k) * np + p, rd);
+#pragma unroll
+        for (int e = 0; e < V; ++e) v[e] = a.dist[k];
+        store_v(out + (size_t)(7 * K + 1 + k) * np + p, v);
+#pragma unroll
+        for (int e = 0; e < V; ++e) v[e] = a.axis[k];
+        store_v(out + (size_t)(8 * K + 1 + k) * np + p, v);
     }
 }
 
@@ -151,12 +202,24 @@ __global__ void __launch_bounds__(256) blend_reduce(const double *__restrict__ p
 
 }  // namespace
 
+namespace {
+
+template <typename OT>
+void launch_features_t(const BlendArgs &a, void *out, cudaStream_t st) {
+    const bool pairs = a.Wt % 2 == 0 && aligned_to(out, 2 * sizeof(OT)) && aligned_to(a.fused, 8) &&
+                       aligned_to(a.rgba, 8) && aligned_to(a.wdepth, 8) && aligned_to(a.alpha, 2);
+    const int v = pairs ? 2 : 1;
+    const dim3 grid((unsigned)((a.Wt + 32 * v - 1) / (32 * v)), (unsigned)((a.Ht + 7) / 8)), block(32, 8);
+    if (pairs) features_kernel<OT, 2><<<grid, block, 0, st>>>(a, reinterpret_cast<OT *>(out));
+    else features_kernel<OT, 1><<<grid, block, 0, st>>>(a, reinterpret_cast<OT *>(out));
+}
+
+}  // namespace
+
 cudaError_t launch_blend_features(const BlendArgs &a, int out_dtype, void *out, cudaStream_t st) {
-    const dim3 grid((unsigned)((a.Wt + 31) / 32), (unsigned)((a.Ht + 7) / 8)), block(32, 8);
-    if (out_dtype == GVS_F16) features_kernel<__half><<<grid, block, 0, st>>>(a, reinterpret_cast<__half *>(out));
-    else if (out_dtype == GVS_BF16)
-        features_kernel<__nv_bfloat16><<<grid, block, 0, st>>>(a, reinterpret_cast<__nv_bfloat16 *>(out));
-    else features_kernel<float><<<grid, block, 0, st>>>(a, reinterpret_cast<float *>(out));
+    if (out_dtype == GVS_F16) launch_features_t<__half>(a, out, st);
+    else if (out_dtype == GVS_BF16) launch_features_t<__nv_bfloat16>(a, out, st);
+    else launch_features_t<float>(a, out, st);
     return cudaGetLastError();
 }
 
