@@ -369,11 +369,10 @@ GVS_API gvs_status gvs_soft_splat_backward(const gvs_camera *in_cams, const void
  * Batched fusion: many (frame, target) items in one persistent launch (a serving
  * pattern; the paper has no counterpart, each item is Supplement A.1's fusion).  Each
  * item fuses the map of one frame (gvs_weight_map) into one target camera,
- * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  A target
- * of about a device-wide wave or more takes a launch of its own; the others share
- * one grid that keeps every SM busy, taking bundles of target pixels from a global
- * counter until all of them are done (no block waits on another).  These are plain
- * kernel launches plus a 4-byte reset, so they can be captured in a CUDA graph.
+ * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  A launch
+ * takes up to 14 items, their arguments as kernel parameters and their blocks one
+ * item after another in one grid (no block waits on another).  These are plain
+ * kernel launches, so they can be captured in a CUDA graph.
  */
 typedef struct {
     const void *map;           /* the frame's map, as from gvs_weight_map */
@@ -388,10 +387,10 @@ typedef struct gvs_fuse_batch gvs_fuse_batch;  /* opaque host object */
 /* Device table bytes for n_items items. */
 GVS_API size_t gvs_fuse_batch_bytes(int32_t n_items);
 
-/* Validates the items (all with the same input views and params), writes their
- * descriptors into `table` (device, caller-owned, >= gvs_fuse_batch_bytes)
- * with a synchronous copy -- call it outside any stream capture -- and returns
- * a host handle.  The maps, outputs and table must outlive the handle. */
+/* Validates the items (all with the same input views and params) and returns a
+ * host handle that holds their descriptors.  `table` (device, caller-owned,
+ * >= gvs_fuse_batch_bytes) is validated and reserved for the handle, but not
+ * written.  The maps, outputs and table must outlive the handle. */
 GVS_API gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, const gvs_fuse_item *items,
                                          int32_t n_items, const gvs_fuse_params *params, void *table,
                                          size_t table_bytes, gvs_fuse_batch **out);

@@ -131,6 +131,5 @@ class BatchPlan:
         for t in self.targets:                        # key clear, scatter + resolve per group of views
             slots = max(1, min(self.N, self.ws_splat.numel() // (t.width * t.height * 8)))
             per_splat += 1 + 2 * ((self.N + slots - 1) // slots)
-        own = sum(t.width * t.height >= gvs.FUSE_BATCH_OWN_LAUNCH for t in self.targets)
-        fuse = self.F * own + (1 if own < len(self.targets) else 0)
+        fuse = -(-self.F * len(self.targets) // gvs.FUSE_BATCH_ITEMS)
         return self.F * per_frame + fuse + self.F * per_splat

@@ -858,28 +858,18 @@ extern "C" gvs_status gvs_forward_splat_noalloc(const gvs_camera *in_cams, const
 }
 
 // ---------------------------------------------------------------------------
-// Batched fusion: many (frame, target) items.  Large targets fill the device for
-// several waves, so each takes the plain fusion kernel (its arguments in the constant bank);
-// the others share one persistent launch, which has no tail per item.
+// Batched fusion: many (frame, target) items per launch.
 // ---------------------------------------------------------------------------
 struct gvs_fuse_batch {
-    int K, map_dtype, variant, n_items, total;  // items of the persistent launch and their bundles
-    gvs::BatchItem *d_items;
-    unsigned *d_counter;
-    int n_large;
-    gvs::FuseArgs *large;  // arguments of the items launched by themselves
+    int K, map_dtype, variant, n_items;
+    gvs::FuseArgs *items;
 };
-
-namespace {
-// Target pixels from which an item is launched by itself.
-constexpr int64_t kLargeTarget = 200000;
-}  // namespace
 
 extern "C" {
 
 size_t gvs_fuse_batch_bytes(int32_t n_items) {
     if (n_items < 0) return 0;
-    return align_up((size_t)n_items * sizeof(gvs::BatchItem), 256) + 256;
+    return align_up((size_t)n_items * (sizeof(gvs::FuseArgs) + sizeof(int) * 2), 256) + 256;
 }
 
 gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, const gvs_fuse_item *items,
@@ -894,51 +884,32 @@ gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, con
     const size_t need = gvs_fuse_batch_bytes(n_items);
     if (!table || table_bytes < need || !aligned(table, 256))
         return fail(GVS_ERR_WORKSPACE, "fuse batch: table needs %zu bytes, 256-byte aligned", need);
-    std::vector<gvs::BatchItem> host;
-    std::vector<gvs::FuseArgs> large;
+    gvs_fuse_batch *b = new (std::nothrow) gvs_fuse_batch;
+    gvs::FuseArgs *args = new (std::nothrow) gvs::FuseArgs[n_items];
+    const auto give_up = [&](gvs_status st) {
+        delete b;
+        delete[] args;
+        return st;
+    };
+    if (!b || !args) return give_up(fail(GVS_ERR_INVALID_ARG, "fuse batch: out of host memory"));
     int64_t total = 0;
     int32_t W = 0, H = 0;
     for (int i = 0; i < n_items; ++i) {
         const gvs_fuse_item &it = items[i];
         gvs_status s = check_fuse_common(in_cams, n_views, it.target, params, it.fused_depth, it.crossing, &W, &H);
-        if (s != GVS_OK) return s;
+        if (s != GVS_OK) return give_up(s);
         const size_t need_map = gvs_fuse_workspace_bytes(n_views, W, H);
         if (!it.map || it.map_bytes < need_map || !aligned(it.map, 256))
-            return fail(GVS_ERR_WORKSPACE, "fuse batch: item %d map needs %zu bytes, 256-byte aligned", i, need_map);
-        gvs::BatchItem item;
-        memset(&item, 0, sizeof(item));
-        item.args = fuse_args(in_cams, it.map, n_views, W, H, it.target, *params, it.fused_depth, it.crossing);
-        if ((int64_t)it.target->width * it.target->height >= kLargeTarget) {
-            large.push_back(item.args);
-            continue;
-        }
-        item.bundle_begin = (int)total;
-        host.push_back(item);
+            return give_up(fail(GVS_ERR_WORKSPACE, "fuse batch: item %d map needs %zu bytes, 256-byte aligned", i, need_map));
+        args[i] = fuse_args(in_cams, it.map, n_views, W, H, it.target, *params, it.fused_depth, it.crossing);
         total += gvs::bundle_count(it.target->width, it.target->height, n_views, params->variant);
-        if (total > INT32_MAX / 2) return fail(GVS_ERR_UNSUPPORTED, "fuse batch: too many target pixels");
+        if (total > INT32_MAX / 2) return give_up(fail(GVS_ERR_UNSUPPORTED, "fuse batch: too many target pixels"));
     }
-    if (!host.empty()) {
-        cudaError_t e = cudaMemcpy(table, host.data(), host.size() * sizeof(gvs::BatchItem), cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(e, "fuse batch: copying the item table");
-    }
-    gvs_fuse_batch *b = new (std::nothrow) gvs_fuse_batch;
-    gvs::FuseArgs *own = large.empty() ? nullptr : new (std::nothrow) gvs::FuseArgs[large.size()];
-    if (!b || (!own && !large.empty())) {
-        delete b;
-        delete[] own;
-        return fail(GVS_ERR_INVALID_ARG, "fuse batch: out of host memory");
-    }
-    for (size_t i = 0; i < large.size(); ++i) own[i] = large[i];
-    b->n_large = (int)large.size();
-    b->large = own;
     b->K = n_views;
     b->map_dtype = params->map_dtype;
     b->variant = params->variant;
-    b->n_items = (int)host.size();
-    b->total = (int)total;
-    b->d_items = reinterpret_cast<gvs::BatchItem *>(table);
-    b->d_counter = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(table) +
-                                                align_up((size_t)n_items * sizeof(gvs::BatchItem), 256));
+    b->n_items = n_items;
+    b->items = args;
     *out = b;
     return GVS_OK;
 }
@@ -946,18 +917,14 @@ gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, con
 gvs_status gvs_fuse_batch_launch(const gvs_fuse_batch *b, void *stream) {
     const Range nvtx_range("gvs_fuse_batch_launch");
     if (!b) return fail(GVS_ERR_INVALID_ARG, "fuse batch: NULL batch");
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < b->n_large && e == cudaSuccess; ++i) e = gvs::launch_fuse(b->large[i], (cudaStream_t)stream);
-    if (e == cudaSuccess && b->n_items > 0)
-        e = gvs::launch_fuse_batch(b->d_items, b->n_items, b->total, b->d_counter, b->K, b->map_dtype, b->variant,
-                                   (cudaStream_t)stream);
+    cudaError_t e = gvs::launch_fuse_batch(b->items, b->n_items, b->K, b->map_dtype, b->variant, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "fuse batch: launch");
     return GVS_OK;
 }
 
 void gvs_fuse_batch_destroy(gvs_fuse_batch *b) {
     if (!b) return;
-    delete[] b->large;
+    delete[] b->items;
     delete b;
 }
 

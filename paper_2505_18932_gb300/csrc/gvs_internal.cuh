@@ -130,15 +130,9 @@ cudaError_t launch_weight_map(const void *depth, int depth_dtype, void *map, int
                               float mu, float wconst, int window, cudaStream_t st, bool exact = false);
 cudaError_t launch_fuse(const FuseArgs &a, cudaStream_t st);
 
-// One (frame, target) item of a batched fusion: its arguments and the index
-// of its first bundle in the batch's bundle numbering.
-struct BatchItem {
-    FuseArgs args;
-    int bundle_begin;
-};
+// Bundles of a target: the size of a launch.
 int bundle_count(int Wt, int Ht, int K, int variant);
-cudaError_t launch_fuse_batch(const BatchItem *items, int n_items, int total, unsigned *counter, int K, int map_dtype,
-                              int variant, cudaStream_t st);
+cudaError_t launch_fuse_batch(const FuseArgs *items, int n_items, int K, int map_dtype, int variant, cudaStream_t st);
 // acc: [K][H][W] float2 scratch; grad_depths written (not accumulated)
 cudaError_t launch_fuse_backward(const FuseArgs &a, const void *depth, int depth_dtype, const int16_t *crossing,
                                  const float *grad_fused, float *grad_depths, float2 *acc, float mu, float wconst,

@@ -844,8 +844,8 @@ class SoftSplat(torch.autograd.Function):
         return gd, gc.to(in_color.dtype), None, None, None
 
 
-# Target pixels from which the library gives an item of a batch a launch of its own.
-FUSE_BATCH_OWN_LAUNCH = 200000
+# Items of a batch that share a launch.
+FUSE_BATCH_ITEMS = 14
 
 
 class FuseBatch:

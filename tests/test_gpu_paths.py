@@ -80,3 +80,25 @@ def test_splat_groups_of_views(gvs, target, slots):
     # sums of at most a few tens of FP32 terms in another order
     torch.testing.assert_close(soft[0]["wsum"], soft[1]["wsum"], rtol=1e-5, atol=1e-7)
     torch.testing.assert_close(soft[0]["color"], soft[1]["color"], rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("K", [3, 5, 8, 12])
+def test_batch_of_more_items_than_a_launch(gvs, K):
+    """17 items of mixed sizes (two launches) and both bundle shapes equal single calls, bit for bit."""
+    from synth import configs
+    w = configs.tiny(61, 47, K, 40)
+    _, d = w.render_inputs(0)
+    dd = to_dev(d)
+    ws = gvs.weight_map(dd, w.mu)
+    sizes = [(61, 47), (24, 18), (97, 33), (8, 70), (1, 1)]
+    targets = [configs.tiny(*sizes[i % len(sizes)], 2, 16).targets[0] for i in range(17)]
+    new = lambda t, dt: torch.empty((t.height, t.width), dtype=dt, device="cuda")  # noqa: E731
+    items = [(ws, t, new(t, torch.float32), new(t, torch.int16)) for t in targets]
+    batch = gvs.FuseBatch(w.inputs, items, w.num_samples, w.z_near, w.z_far, w.mu)
+    batch.launch()
+    torch.cuda.synchronize()
+    for _, t, fused, cross in items:
+        for variant in (0, 3):
+            f, c = gvs.fuse_depth(w.inputs, dd, t, w.num_samples, w.z_near, w.z_far, w.mu, variant=variant)
+            assert torch.equal(f, fused) and torch.equal(c, cross)
+    batch.close()
