@@ -427,10 +427,11 @@ int bundle_count(int Wt, int Ht, int K, int variant) {
 }
 
 cudaError_t launch_fuse(const FuseArgs &a, cudaStream_t st) {
+    const int64_t target = (int64_t)a.Wt * a.Ht, view = (int64_t)a.W * a.H;
     if (a.tmp_depth || a.wview)
-        by_kmax_tile0<FuseLaunchTemporal>(a.K, a.map_dtype, a, st);
+        by_kmax_tile0<FuseLaunchTemporal>(a.K, a.map_dtype, shaped_variant(0, a.K, target, view), a, st);
     else
-        by_kmax<FuseLaunch>(a.K, a.map_dtype, a.variant, a, st);
+        by_kmax<FuseLaunch>(a.K, a.map_dtype, shaped_variant(a.variant, a.K, target, view), a, st);
     return cudaGetLastError();
 }
 

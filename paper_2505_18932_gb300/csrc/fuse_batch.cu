@@ -53,6 +53,10 @@ struct BatchLaunch {
 }  // namespace
 
 cudaError_t launch_fuse_batch(const FuseArgs *items, int n_items, int K, int map_dtype, int variant, cudaStream_t st) {
+    // one bundle shape for the launch: the one that suits the items' mean size
+    int64_t pixels = 0;
+    for (int i = 0; i < n_items; ++i) pixels += (int64_t)items[i].Wt * items[i].Ht;
+    variant = shaped_variant(variant, K, pixels, (int64_t)n_items * items[0].W * items[0].H);
     by_kmax<BatchLaunch>(K, map_dtype, variant, items, n_items, st);
     return cudaGetLastError();
 }

@@ -128,6 +128,14 @@ constexpr int fuse_min_blocks() {
     return KMAX <= 4 ? 7 : (T::full && !T::warp && !TMP && KMAX <= 16) ? 12 : 9;
 }
 
+// The bundle shape of the default variant 0.  Up to 8 views, 4 x 8 pixels (as variant 3) beats
+// 8 x 4 unless the target is much coarser than the views (us, 8 x 4 and 4 x 8: 8 x 1080p 236 and
+// 227, 5 x 961x541 68 and 62, 7 x 720p arc 122 and 109, 4 x 640x360 27 and 23, temporal 720p
+// 146 and 144; 8 x 720p into 640x360 71 and 75); for more views the two are level.
+inline int shaped_variant(int variant, int K, int64_t target_pixels, int64_t view_pixels) {
+    return variant == 0 && K <= 8 && 2 * target_pixels >= view_pixels ? 3 : variant;
+}
+
 struct Ray {
     float ax, ay, az;
 };
@@ -654,8 +662,9 @@ __device__ __forceinline__ void march_bundle(const FuseArgs &a, const int2 *tab,
 
 // Calls F<Tile_i>::run(...) for the variant, with the full form of the tile
 // when the call has exactly KMAX views; views counts other than 8 and 16 use
-// the default tile only (fewer instantiations to build), except the
-// warp-per-ray variant 6, built for 8, 16 and 32 views (5 to 32 views).
+// the default tile only (fewer instantiations to build), except the 4 x 8
+// bundles of up to 4 views and the warp-per-ray variant 6, built for 8, 16 and
+// 32 views (5 to 32 views).
 template <int KMAX, typename MT, template <int, typename, typename> class F, typename T, typename... Args>
 void full_or_not(int K, Args... args) {
     if (K == KMAX) F<KMAX, MT, typename FullTile<T>::type>::run(args...);
@@ -680,6 +689,10 @@ void by_variant(int K, int variant, Args... args) {
             default: break;
         }
     }
+    if (KMAX == 4 && variant == 3) {
+        full_or_not<KMAX, MT, F, Tile3>(K, args...);
+        return;
+    }
     full_or_not<KMAX, MT, F, Tile0>(K, args...);
 }
 
@@ -698,19 +711,25 @@ void by_kmax(int K, int map_dtype, int variant, Args... args) {
     }
 }
 
-// The same for kernels built with the default tile only.
+// The same for kernels built with the default variant's tiles only (variant 3: the 4 x 8 one).
+template <int KMAX, typename MT, template <int, typename, typename> class F, typename... Args>
+void by_shape(int K, int variant, Args... args) {
+    if (KMAX <= 8 && variant == 3) full_or_not<KMAX, MT, F, Tile3>(K, args...);
+    else full_or_not<KMAX, MT, F, Tile0>(K, args...);
+}
+
 template <template <int, typename, typename> class F, typename... Args>
-void by_kmax_tile0(int K, int map_dtype, Args... args) {
+void by_kmax_tile0(int K, int map_dtype, int variant, Args... args) {
     if (map_dtype == GVS_F16) {
-        if (K <= 4) full_or_not<4, __half2, F, Tile0>(K, args...);
-        else if (K <= 8) full_or_not<8, __half2, F, Tile0>(K, args...);
-        else if (K <= 16) full_or_not<16, __half2, F, Tile0>(K, args...);
-        else full_or_not<32, __half2, F, Tile0>(K, args...);
+        if (K <= 4) by_shape<4, __half2, F>(K, variant, args...);
+        else if (K <= 8) by_shape<8, __half2, F>(K, variant, args...);
+        else if (K <= 16) by_shape<16, __half2, F>(K, variant, args...);
+        else by_shape<32, __half2, F>(K, variant, args...);
     } else {
-        if (K <= 4) full_or_not<4, float2, F, Tile0>(K, args...);
-        else if (K <= 8) full_or_not<8, float2, F, Tile0>(K, args...);
-        else if (K <= 16) full_or_not<16, float2, F, Tile0>(K, args...);
-        else full_or_not<32, float2, F, Tile0>(K, args...);
+        if (K <= 4) by_shape<4, float2, F>(K, variant, args...);
+        else if (K <= 8) by_shape<8, float2, F>(K, variant, args...);
+        else if (K <= 16) by_shape<16, float2, F>(K, variant, args...);
+        else by_shape<32, float2, F>(K, variant, args...);
     }
 }
 
