@@ -38,7 +38,8 @@ namespace {
 // group's terms to S_s and S_{s+1} in view order (the forward's own order and
 // operations, so the same bits) and, with its terms still in registers, issues its two
 // atomics.  8 x 1080p: 121 -> 107 us against a thread to a pixel, which recomputed every
-// term after the sums; resident blocks 8 (64 registers), 12, 16: 107, 115, 112 us.
+// term after the sums; resident blocks 8 (64 registers), 12, 16: 107, 115, 112 us.  The list
+// carries each pixel's sample and gradient, one load less in the chain: 96 us.
 constexpr int BS_TX = 16, BS_TY = 32, BS_THREADS = 128, BS_BLOCKS = 8;
 template <int KMAX, typename MT>
 __global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const __grid_constant__ FuseArgs a,
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const 
                                                                          float2 *__restrict__ acc) {
     constexpr int PER = BS_TX * BS_TY / BS_THREADS;  // pixels per thread in the listing pass
     constexpr int GROUPS = BS_THREADS / KMAX;        // pixels at a time
-    __shared__ int s_list[BS_TX * BS_TY];
+    __shared__ int2 s_list[BS_TX * BS_TY];  // (tile-local raster index | sample << 16, upstream gradient)
     __shared__ int s_warp[BS_THREADS / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int base = 0;
@@ -55,12 +56,14 @@ __global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const 
     for (int r = 0; r < PER; ++r) {
         const int e = r * BS_THREADS + tid;  // tile-local raster index
         const int i = blockIdx.x * BS_TX + (e % BS_TX), j = blockIdx.y * BS_TY + (e / BS_TX);
-        bool work = false;
+        int s = -1;
+        float G = 0.0f;
         if (i < a.Wt && j < a.Ht) {
             const size_t o = (size_t)j * a.Wt + i;
-            const int s = crossing[o];
-            work = s >= 0 && s + 1 < a.D && grad_fused[o] != 0.0f;
+            s = crossing[o];
+            G = grad_fused[o];
         }
+        const bool work = s >= 0 && s + 1 < a.D && G != 0.0f;
         const unsigned ball = __ballot_sync(0xffffffffu, work);
         if (lane == 0) s_warp[warp] = __popc(ball);
         __syncthreads();
@@ -68,7 +71,8 @@ __global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const 
         for (int w = 0; w < warp; ++w) before += s_warp[w];
         int total = base;
         for (int w = 0; w < BS_THREADS / 32; ++w) total += s_warp[w];
-        if (work) s_list[before + __popc(ball & ((1u << lane) - 1u))] = e;
+        if (work)  // a sample index has 15 bits, a tile index 9
+            s_list[before + __popc(ball & ((1u << lane) - 1u))] = make_int2(e | (s << 16), __float_as_int(G));
         __syncthreads();  // s_warp is rewritten by the next round
         base = total;
     }
@@ -80,11 +84,10 @@ __global__ void __launch_bounds__(BS_THREADS, BS_BLOCKS) fuse_bwd_scatter(const 
     for (int q0 = warp * (32 / KMAX); q0 < base; q0 += GROUPS) {  // the same for the whole warp
         const int q = q0 + lane / KMAX;
         const bool on = q < base;
-        const int e = s_list[on ? q : q0];
+        const int2 l = s_list[on ? q : q0];
+        const int e = l.x & 0xffff, s = l.x >> 16;
+        const float G = __int_as_float(l.y);
         const int i = blockIdx.x * BS_TX + (e % BS_TX), j = blockIdx.y * BS_TY + (e / BS_TX);
-        const size_t o = (size_t)j * a.Wt + i;
-        const int s = crossing[o];
-        const float G = grad_fused[o];
         const float fi = (float)i, fj = (float)j;
         const float ax = __fmaf_rn(xf.M[0], fi, __fmaf_rn(xf.M[1], fj, xf.M[2]));
         const float ay = __fmaf_rn(xf.M[3], fi, __fmaf_rn(xf.M[4], fj, xf.M[5]));
