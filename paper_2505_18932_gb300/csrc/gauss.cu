@@ -196,8 +196,37 @@ __global__ void __launch_bounds__(256) gauss_fill(const GaussArgs g) {
     const unsigned long long *off = reinterpret_cast<const unsigned long long *>(g.ws + g.L.off_offset);
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(g.ws + g.L.off_keys);
     const unsigned long long key = ((unsigned long long)__float_as_uint(a.z) << 32) | (unsigned)src;
-    for (int ty = j0 / GS_TILE; ty <= j1 / GS_TILE; ++ty)
-        for (int tx = i0 / GS_TILE; tx <= i1 / GS_TILE; ++tx) {
+    const int tx0 = i0 / GS_TILE, tx1 = i1 / GS_TILE, ty0 = j0 / GS_TILE, ty1 = j1 / GS_TILE;
+    if (tx1 - tx0 <= 1 && ty1 - ty0 <= 1) {
+        // the usual box: at most 2 x 2 tiles, whose counters answer together (4 views at 720p:
+        // 57 -> 52 us)
+        unsigned base[4], peers[4];
+        unsigned long long first[4];
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int tx = tx0 + (e & 1), ty = ty0 + (e >> 1);
+            peers[e] = 0u;
+            if (tx <= tx1 && ty <= ty1) {
+                const int t = ty * g.L.tiles_x + tx;
+                peers[e] = __match_any_sync(__activemask(), t);
+                base[e] = 0u;
+                first[e] = off[t];
+                if (lane == __ffs(peers[e]) - 1) base[e] = atomicAdd(&cursor[t], (unsigned)__popc(peers[e]));
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (peers[e]) {
+                const unsigned b = __shfl_sync(peers[e], base[e], __ffs(peers[e]) - 1);
+                const unsigned long long pos = first[e] + b + __popc(peers[e] & ((1u << lane) - 1u));
+                if (GVS_IN_BOUNDS(pos, g.L.n_keys, GVS_SITE_GAUSS_KEY)) keys[pos] = key;
+            }
+        }
+        return;
+    }
+    for (int ty = ty0; ty <= ty1; ++ty)
+        for (int tx = tx0; tx <= tx1; ++tx) {
             const int t = ty * g.L.tiles_x + tx;
             const unsigned long long pos = off[t] + agg_increment(cursor, t);
             if (GVS_IN_BOUNDS(pos, g.L.n_keys, GVS_SITE_GAUSS_KEY)) keys[pos] = key;
