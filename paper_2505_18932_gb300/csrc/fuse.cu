@@ -11,7 +11,7 @@
 // depth_bounds, bounds_overlap: build the per-view bound pyramid (16, 32, 64
 //               and 128 pixel tiles, each also as overlapping 2x2-tile
 //               blocks, and the whole view) from the 16x16 tiles.
-// fuse        : one warp per 8x4 bundle of target pixels, one thread per ray,
+// fuse        : one warp per bundle of 32 target pixels (4x8 or 8x4), one thread per ray,
 //               marching the D samples in registers (one 8-byte gather per
 //               sample and view) to the first +/- crossing.  Before evaluating
 //               samples the warp tries to prove that a run of them holds no

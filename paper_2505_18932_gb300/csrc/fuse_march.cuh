@@ -118,14 +118,14 @@ constexpr int kFuseVariants = 7;
 // Resident blocks per SM asked of the register allocator, measured over 5 to 12 (us):
 //   8 or 16 views, all of them present: 12 (40 registers; the rays spill to L1 and the warps
 //     hide it): 8 x 1080p 254 against 274 at 9 and 301 at 7; 16 x 1080p, half2 map, 507
-//     against 557 and 621;
+//     against 557 and 621 (one view per step; two: 236 and 467 at 12);
 //   up to 4 views: 7 (72 registers), for small targets are one wave of bundles whose time is
 //     one bundle's chain of tests and samples: 4 x 320x240 26.8 against 28.8 at 9;
-//   otherwise (a guard per view, the temporal input, 32 views): 9 (56 registers):
-//     5 views at 961x541 68.0 against 71.7 at 12 and 71.5 at 7.
+//   otherwise (exactly 5 to 7 views, a guard per view, the temporal input, 32 views): 9
+//     (56 registers): 5 views at 961x541 49.6 against 51.0 at 12.
 template <int KMAX, typename T, bool TMP>
 constexpr int fuse_min_blocks() {
-    return KMAX <= 4 ? 7 : (T::full && !T::warp && !TMP && KMAX <= 16) ? 12 : 9;
+    return KMAX <= 4 ? 7 : (T::full && !T::warp && !TMP && KMAX >= 8 && KMAX <= 16) ? 12 : 9;
 }
 
 // The bundle shape of the default variant 0.  Up to 8 views, 4 x 8 pixels (as variant 3) beats
@@ -281,8 +281,7 @@ __device__ __forceinline__ bool slab_view_free(const FuseArgs &a, const int2 *ta
 template <int KMAX, typename MT, bool FULL = false, bool PLANES = true>
 __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&ray)[KMAX], float zs, float &S,
                                                 float &Wsum) {
-    constexpr int G = !FULL ? 1 : KMAX <= 4 ? 4 : 2;
-    static_assert(KMAX % G == 0, "whole groups");
+    constexpr int G = !FULL ? 1 : KMAX <= 4 ? KMAX : 2;
     const size_t plane = (size_t)a.W * a.H;
     S = 0.0f;
     Wsum = 0.0f;
@@ -295,6 +294,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 const int k = k0 + g;
+                if (k >= KMAX) continue;
                 hz[g] = __fmaf_rn(zs, ray[k].az, a.xf[k].b[2]);
                 const float hx = __fmaf_rn(zs, ray[k].ax, a.xf[k].b[0]);
                 const float hy = __fmaf_rn(zs, ray[k].ay, a.xf[k].b[1]);
@@ -304,6 +304,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
                     const int k = k0 + g;
+                    if (k >= KMAX) continue;
                     nearest_pixel_exact(__fmaf_rn(zs, ray[k].ax, a.xf[k].b[0]),
                                         __fmaf_rn(zs, ray[k].ay, a.xf[k].b[1]), hz[g], u[g], v[g]);
                 }
@@ -313,6 +314,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
 #pragma unroll
             for (int g = 0; g < G; ++g) {
                 const int k = k0 + g;
+                if (k >= KMAX) continue;
                 in[g] = hz[g] > 1e-6f && (unsigned)u[g] < (unsigned)a.W && (unsigned)v[g] < (unsigned)a.H &&
                         GVS_IN_BOUNDS((size_t)k * plane + (size_t)v[g] * a.W + u[g], (size_t)a.K * plane,
                                       GVS_SITE_FUSE_MAP);
@@ -325,6 +327,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
             }
 #pragma unroll
             for (int g = 0; g < G; ++g) {
+                if (k0 + g >= KMAX) continue;
                 const float sdf = (p[g].x - hz[g]) * a.inv_mu;
                 const float w = (in[g] && sdf >= -1.0f) ? p[g].y : 0.0f;
                 S = fmaf(w, fminf(sdf, 1.0f), S);
@@ -696,14 +699,33 @@ void by_variant(int K, int variant, Args... args) {
     full_or_not<KMAX, MT, F, Tile0>(K, args...);
 }
 
+// View counts below 8 that are not a power of two: kernels for exactly K views (4 x 8
+// bundles).  A slab test takes 32 / K segments of K lanes, and no view has a guard:
+// 5 x 961x541 63 -> 50 us, 7 x 720p arc 109 -> 98 (9 blocks per SM; 12: 51 and 99).
+template <typename MT, template <int, typename, typename> class F, typename... Args>
+bool by_exact_k(int K, int variant, Args... args) {
+    if (variant != 3) return false;
+    using T = typename FullTile<Tile3>::type;
+    switch (K) {
+        case 2: F<2, MT, T>::run(args...); return true;
+        case 3: F<3, MT, T>::run(args...); return true;
+        case 5: F<5, MT, T>::run(args...); return true;
+        case 6: F<6, MT, T>::run(args...); return true;
+        case 7: F<7, MT, T>::run(args...); return true;
+        default: return false;
+    }
+}
+
 template <template <int, typename, typename> class F, typename... Args>
 void by_kmax(int K, int map_dtype, int variant, Args... args) {
     if (map_dtype == GVS_F16) {
+        if (by_exact_k<__half2, F>(K, variant, args...)) return;
         if (K <= 4) by_variant<4, __half2, F>(K, variant, args...);
         else if (K <= 8) by_variant<8, __half2, F>(K, variant, args...);
         else if (K <= 16) by_variant<16, __half2, F>(K, variant, args...);
         else by_variant<32, __half2, F>(K, variant, args...);
     } else {
+        if (by_exact_k<float2, F>(K, variant, args...)) return;
         if (K <= 4) by_variant<4, float2, F>(K, variant, args...);
         else if (K <= 8) by_variant<8, float2, F>(K, variant, args...);
         else if (K <= 16) by_variant<16, float2, F>(K, variant, args...);
@@ -720,6 +742,7 @@ void by_shape(int K, int variant, Args... args) {
 
 template <template <int, typename, typename> class F, typename... Args>
 void by_kmax_tile0(int K, int map_dtype, int variant, Args... args) {
+    if (map_dtype != GVS_F16 && by_exact_k<float2, F>(K, variant, args...)) return;
     if (map_dtype == GVS_F16) {
         if (K <= 4) by_shape<4, __half2, F>(K, variant, args...);
         else if (K <= 8) by_shape<8, __half2, F>(K, variant, args...);

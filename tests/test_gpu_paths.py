@@ -9,6 +9,7 @@ from gpu_util import to_dev, u32
 from test_gpu_gauss import _case as gauss_case
 from test_gpu_grad import _case as grad_case
 from test_gpu_slab import _rig
+from test_gpu_slab import test_slab_on_turned_views as turned_views
 
 pytestmark = pytest.mark.gpu
 
@@ -82,7 +83,7 @@ def test_splat_groups_of_views(gvs, target, slots):
     torch.testing.assert_close(soft[0]["color"], soft[1]["color"], rtol=1e-5, atol=1e-5)
 
 
-@pytest.mark.parametrize("K", [3, 5, 8, 12])
+@pytest.mark.parametrize("K", [2, 3, 5, 6, 7, 8, 12])
 def test_batch_of_more_items_than_a_launch(gvs, K):
     """17 items of mixed sizes (two launches) and both bundle shapes equal single calls, bit for bit."""
     from synth import configs
@@ -98,7 +99,13 @@ def test_batch_of_more_items_than_a_launch(gvs, K):
     batch.launch()
     torch.cuda.synchronize()
     for _, t, fused, cross in items:
-        for variant in (0, 3):
+        for variant in (0, 1, 3):
             f, c = gvs.fuse_depth(w.inputs, dd, t, w.num_samples, w.z_near, w.z_far, w.mu, variant=variant)
             assert torch.equal(f, fused) and torch.equal(c, cross)
     batch.close()
+
+
+@pytest.mark.parametrize("n,size,samples", [(2, (61, 47), 96), (6, (61, 47), 64), (7, (40, 33), 33)])
+def test_fuse_of_exact_view_counts(gvs, oracle_mod, n, size, samples):
+    """Counts of views with a kernel of their own, on turned views, against the oracle."""
+    turned_views(gvs, oracle_mod, n, size, samples, (0, 1, 3))
