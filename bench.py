@@ -844,7 +844,7 @@ def mixed_form(device, steps, pixels=2048):
 
 def time_batched(device, steps):
     """The serving-style workload (8 x 1280x720 inputs, 16 targets of four sizes, 2 frames):
-    the CUDA-graph BatchPlan (one persistent fusion launch, autotuned variant) against the
+    the CUDA-graph BatchPlan (fusion in shared launches, autotuned variant) against the
     same work through the single-view API, launched eagerly item by item."""
     import torch
     from paper_2505_18932_gb300 import batch, gvs
@@ -856,7 +856,7 @@ def time_batched(device, steps):
     plan = batch.BatchPlan(w.inputs, w.targets, rgba[1:], dep[1:], w.num_samples, w.z_near, w.z_far, w.mu,
                            tau=w.tau, rgba_prev=rgba[0], state0=dep[0], variant=None, graph=True)
     graph_ms = _event_ms(plan.run, steps)
-    # the same launch sequence without the graph: refine, maps, one persistent fusion, 32 splats
+    # the same launch sequence without the graph: refine, maps, shared fusion launches, 32 splats
     same_ms = _event_ms(plan._run_eager, steps)
 
     def per_item():
@@ -879,8 +879,8 @@ def time_batched(device, steps):
                               "value": round(px / (graph_ms * 1e-3) / 1e6, 3), "unit": "target Mpix/s",
                               "variant": plan.variant, "autotune_ms": plan.timings,
                               "launches_per_step": plan.launches_per_run(),
-                              "note": "2 frames x 16 targets (640x360 .. 1920x1080): refine + maps + one persistent "
-                                      "fusion + 32 splats, replayed as one CUDA graph"},
+                              "note": "2 frames x 16 targets (640x360 .. 1920x1080): refine + maps + shared fusion "
+                                      "launches + 32 splats, replayed as one CUDA graph"},
             "batched_eager_same_launches": {"ms_per_step": round(same_ms, 4), "steps": steps, "workload": w.name,
                                             "value": round(px / (same_ms * 1e-3) / 1e6, 3), "unit": "target Mpix/s",
                                             "note": "the graph's launch sequence issued eagerly"},

@@ -366,7 +366,7 @@ GVS_API gvs_status gvs_soft_splat_backward(const gvs_camera *in_cams, const void
                                            float *grad_in_depth, float *grad_in_color, void *stream);
 
 /*
- * Batched fusion: many (frame, target) items in one persistent launch (a serving
+ * Batched fusion: many (frame, target) items in shared launches (a serving
  * pattern; the paper has no counterpart, each item is Supplement A.1's fusion).  Each
  * item fuses the map of one frame (gvs_weight_map) into one target camera,
  * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  A launch

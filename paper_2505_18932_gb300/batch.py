@@ -3,8 +3,8 @@ many target views of uneven size, as one CUDA graph.
 
 Per frame f (in order, each refining against the previous frame):
     refine_depth -> weight_map            (one map per frame)
-then ONE persistent launch fuses every (frame, target) item
-    gvs_fuse_batch_launch                 (bundles pulled from a global counter)
+then one launch per 14 (frame, target) items fuses them all
+    gvs_fuse_batch_launch                 (the items' blocks one after another)
 and every (frame, target) pair is splatted with the fused depth as guide
     forward_splat.
 The whole sequence is captured once into a torch.cuda.CUDAGraph and replayed

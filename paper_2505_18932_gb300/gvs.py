@@ -849,7 +849,7 @@ FUSE_BATCH_ITEMS = 14
 
 
 class FuseBatch:
-    """Batched fusion of many (map, target) items in one persistent launch (gvs_fuse_batch_*).
+    """Batched fusion of many (map, target) items in shared launches (gvs_fuse_batch_*).
 
     items: list of (map_tensor, target_camera, fused_out [Ht, Wt] float32, crossing_out int16 or None).
     Create outside any stream capture (it copies the item table); launch() may be captured."""
