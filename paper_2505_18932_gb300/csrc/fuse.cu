@@ -35,6 +35,44 @@ __device__ __forceinline__ unsigned shl_sat(unsigned x, unsigned n) {
     return r;
 }
 
+// The taps of one row of the tile, `src` its first value of the thread's window: row r of
+// the WM_P + 2R a thread reads belongs to the windows of outputs r - 2R .. r.  ALL: every output's.
+// Two vertically adjacent outputs take a neighbour they share in one packed
+// add and one packed FMA: |dc - n| = |n + (-dc)| exactly, and each output
+// sums its taps in raster order with the same roundings.
+// Windows above 9 x 9 take the rows of every output in a rolled loop.  With all rows unrolled,
+// the compiler (13.0) spilled hundreds of bytes of packed pairs at 32 registers and the 13 x 13
+// and 15 x 15 sums came out up to 11 % off; the same loop with scalar operations, or with registers
+// for all pairs, was right, so the weights must not hang on how a fully unrolled loop spills.  8 x 1080p,
+// windows 11, 13, 15: 211, 272, 344 us, against 228, 284, 365 unrolled with 64 registers.
+template <int R, bool ALL>
+__device__ __forceinline__ void row_taps(const float2 *src, int r, float mu, const float2 (&ndc)[WM_P / 2],
+                                         float2 (&nu)[WM_P / 2]) {
+    float2 row[2 * R + 1];
+#pragma unroll
+    for (int dx = 0; dx <= 2 * R; ++dx) row[dx] = src[dx];
+#pragma unroll
+    for (int q = 0; q < WM_P / 2; ++q) {
+        const bool in0 = ALL || (r - 2 * q >= 0 && r - 2 * q <= 2 * R);
+        const bool in1 = ALL || (r - 2 * q - 1 >= 0 && r - 2 * q - 1 <= 2 * R);
+#pragma unroll
+        for (int dx = 0; dx <= 2 * R; ++dx) {
+            // fminf returns mu for a NaN (invalid) neighbour: it counts mu^2
+            if (in0 && in1) {
+                const float2 e = __fadd2_rn(row[dx], ndc[q]);
+                const float2 t = make_float2(fminf(fabsf(e.x), mu), fminf(fabsf(e.y), mu));
+                nu[q] = __ffma2_rn(t, t, nu[q]);
+            } else if (in0) {
+                const float t = fminf(fabsf(row[dx].x + ndc[q].x), mu);
+                nu[q].x = fmaf(t, t, nu[q].x);
+            } else if (in1) {
+                const float t = fminf(fabsf(row[dx].y + ndc[q].y), mu);
+                nu[q].y = fmaf(t, t, nu[q].y);
+            }
+        }
+    }
+}
+
 // R = window / 2.  The shared tile holds the block's depths, as the map will
 // store them, plus an R-pixel halo replicated at the image borders (invalid
 // depths as NaN).  A thread reads each of the (WM_P + 2R) x (2R + 1) shared
@@ -44,12 +82,11 @@ __device__ __forceinline__ unsigned shl_sat(unsigned x, unsigned n) {
 // operations (bit-reproducible on the host, as the sphere-tracing path needs);
 // otherwise with the approximate reciprocal square root.
 // 8 resident blocks per SM (32 registers): the stencil needs the warps more
-// than the registers (at 51 registers 10 % slower).  8 x 1080p: 122 -> 119 us since the
+// than the registers (8 x 1080p, windows 7, 9, 11, 13, 15: 123, 164, 211, 272, 344 us; with
+// 4 blocks of 64 registers 147, 176, 219, 277, 351).  8 x 1080p: 122 -> 119 us since the
 // epilogue tests nothing per pixel where a warp's pixels are all valid.
-// Windows above 9 x 9 get 64 registers: at 32 they spill hundreds of bytes, and the 15 x 15
-// kernel then summed wrong terms for the first output of each thread.
 template <int R, typename DT, typename MT, bool EXACT = false>
-__global__ void __launch_bounds__(256, R <= 4 ? 8 : 4) weight_map_kernel(const DT *__restrict__ depth, char *__restrict__ map,
+__global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict__ depth, char *__restrict__ map,
                                                          MapLayout L, float mu, float wconst, float inv_w2) {
     constexpr int SW = WM_TX + 2 * R;
     constexpr int SH = WM_TY + 2 * R;
@@ -91,9 +128,6 @@ __global__ void __launch_bounds__(256, R <= 4 ? 8 : 4) weight_map_kernel(const D
     __syncthreads();
     const int x = blockIdx.x * WM_TX + tx;
     const int yb = blockIdx.y * WM_TY + ty * WM_P;
-    // Two vertically adjacent outputs take a neighbour they share in one packed
-    // add and one packed FMA: |dc - n| = |n + (-dc)| exactly, and each output
-    // still sums its taps in the same order with the same roundings.
     static_assert(WM_P % 2 == 0, "outputs are paired");
     float2 ndc[WM_P / 2], nu[WM_P / 2];  // -dc and nu of each pair
 #pragma unroll
@@ -101,31 +135,17 @@ __global__ void __launch_bounds__(256, R <= 4 ? 8 : 4) weight_map_kernel(const D
         ndc[q] = make_float2(-tile[ty * WM_P + 2 * q + R][tx + R].x, -tile[ty * WM_P + 2 * q + 1 + R][tx + R].x);
         nu[q] = make_float2(0.0f, 0.0f);
     }
+    const float2(*rows)[SW] = &tile[ty * WM_P];
+    if (R <= 4) {
 #pragma unroll
-    for (int r = 0; r < WM_P + 2 * R; ++r) {
-        float2 row[2 * R + 1];
+        for (int r = 0; r < WM_P + 2 * R; ++r) row_taps<R, false>(&rows[r][tx], r, mu, ndc, nu);
+    } else {
 #pragma unroll
-        for (int dx = 0; dx <= 2 * R; ++dx) row[dx] = tile[ty * WM_P + r][tx + dx];
+        for (int r = 0; r < WM_P - 1; ++r) row_taps<R, false>(&rows[r][tx], r, mu, ndc, nu);
+#pragma unroll 1
+        for (int r = WM_P - 1; r <= 2 * R; ++r) row_taps<R, true>(&rows[r][tx], r, mu, ndc, nu);
 #pragma unroll
-        for (int q = 0; q < WM_P / 2; ++q) {
-            const bool in0 = r - 2 * q >= 0 && r - 2 * q <= 2 * R;
-            const bool in1 = r - 2 * q - 1 >= 0 && r - 2 * q - 1 <= 2 * R;
-#pragma unroll
-            for (int dx = 0; dx <= 2 * R; ++dx) {
-                // fminf returns mu for a NaN (invalid) neighbour: it counts mu^2
-                if (in0 && in1) {
-                    const float2 e = __fadd2_rn(row[dx], ndc[q]);
-                    const float2 t = make_float2(fminf(fabsf(e.x), mu), fminf(fabsf(e.y), mu));
-                    nu[q] = __ffma2_rn(t, t, nu[q]);
-                } else if (in0) {
-                    const float t = fminf(fabsf(row[dx].x + ndc[q].x), mu);
-                    nu[q].x = fmaf(t, t, nu[q].x);
-                } else if (in1) {
-                    const float t = fminf(fabsf(row[dx].y + ndc[q].y), mu);
-                    nu[q].y = fmaf(t, t, nu[q].y);
-                }
-            }
-        }
+        for (int r = 2 * R + 1; r < WM_P + 2 * R; ++r) row_taps<R, false>(&rows[r][tx], r, mu, ndc, nu);
     }
     float nd[WM_P];  // -dc, NaN where there is no valid pixel
 #pragma unroll
