@@ -118,11 +118,12 @@ typedef struct {
     int32_t depth_dtype;       /* GVS_F32 or GVS_F16: element type of in_depths */
     int32_t map_dtype;         /* GVS_F32: (d, omega) as float2; GVS_F16: as half2 (omega rounded to half) */
     int32_t variant;           /* 0..6: mapping, bundle shape, slab-test lengths and samples evaluated at
-                                  once by the march (lane per ray: 0: 8x4, 1: 8x4 longer segments, 2: 16x2,
-                                  3: 4x8, 4: 4x8 and 5: 8x4 with two samples at once, for 5..16 views;
-                                  warp per ray: 6, its lanes over views x consecutive samples, for 5..32
-                                  views); other view counts run variant 0.  Every variant gives the same
-                                  result, the autotuner picks the fastest (0 = default) */
+                                  once by the march.  0 (default): a ray per lane in bundles of 8x4 or
+                                  4x8 pixels, by views and sizes.  For 5..16 views 1: 8x4 (where 0 is
+                                  8x4: with longer segments), 2: 16x2, 3: 4x8, 4: 4x8 and 5: 8x4 with two
+                                  samples at once.  For 5..32 views 6: a ray per warp, its lanes over
+                                  views x consecutive samples.  Otherwise as 0.  Every variant gives the
+                                  same result, the autotuner picks the fastest */
 } gvs_fuse_params;
 
 /* Forward splat (Sec. 3.1, Supplement A.3). */

@@ -23,12 +23,15 @@ VARIANTS = (0, 1, 2, 3, 4, 5, 6)
 _lock = threading.Lock()
 
 
-def variants_for(n_views: int):
+def variants_for(n_views: int, target_pixels: int = None, view_pixels: int = None):
     """The variants that are distinct kernels for a call with n_views input views: the
-    lane-per-ray bundle shapes (0..5) are compiled for 5..16 views (8- and 16-view
-    kernels), the warp-per-ray mapping (6) for 5..32 views; otherwise a variant runs the
-    default shape."""
+    lane-per-ray bundle shapes (0..5) are compiled for 5..16 views, the warp-per-ray mapping
+    (6) for 5..32 views; otherwise a variant runs the default shape.  With the pixels of the
+    target and of a view given, 3 is left out where the default already is that shape (see
+    shaped_variant in csrc/gvs_internal.cuh)."""
     if 5 <= n_views <= 16:
+        if n_views <= 8 and target_pixels is not None and 2 * target_pixels >= view_pixels:
+            return tuple(v for v in VARIANTS if v != 3)
         return VARIANTS
     return (0, 6) if n_views > 16 else (0,)
 

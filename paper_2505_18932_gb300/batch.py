@@ -85,7 +85,9 @@ class BatchPlan:
         def runner(v):
             batches[v] = self._make_batch(v)
             return batches[v].launch
-        best, timings = autotune.choose(shape, runner, candidates=autotune.variants_for(len(self.cams)))
+        mean = sum(t.width * t.height for t in self.targets) / len(self.targets)
+        candidates = autotune.variants_for(self.N, mean, self.shape[1] * self.shape[2])
+        best, timings = autotune.choose(shape, runner, candidates=candidates)
         for b in batches.values():
             b.close()
         return best, timings

@@ -128,14 +128,6 @@ constexpr int fuse_min_blocks() {
     return KMAX <= 4 ? 7 : (T::full && !T::warp && !TMP && KMAX >= 8 && KMAX <= 16) ? 12 : 9;
 }
 
-// The bundle shape of the default variant 0.  Up to 8 views, 4 x 8 pixels (as variant 3) beats
-// 8 x 4 unless the target is much coarser than the views (us, 8 x 4 and 4 x 8: 8 x 1080p 236 and
-// 227, 5 x 961x541 68 and 62, 7 x 720p arc 122 and 109, 4 x 640x360 27 and 23, temporal 720p
-// 146 and 144; 8 x 720p into 640x360 71 and 75); for more views the two are level.
-inline int shaped_variant(int variant, int K, int64_t target_pixels, int64_t view_pixels) {
-    return variant == 0 && K <= 8 && 2 * target_pixels >= view_pixels ? 3 : variant;
-}
-
 struct Ray {
     float ax, ay, az;
 };
@@ -664,10 +656,9 @@ __device__ __forceinline__ void march_bundle(const FuseArgs &a, const int2 *tab,
 }
 
 // Calls F<Tile_i>::run(...) for the variant, with the full form of the tile
-// when the call has exactly KMAX views; views counts other than 8 and 16 use
-// the default tile only (fewer instantiations to build), except the 4 x 8
-// bundles of up to 4 views and the warp-per-ray variant 6, built for 8, 16 and
-// 32 views (5 to 32 views).
+// when the call has exactly KMAX views.  The 8- and 16-view kernels (5 to 16 views)
+// have every tile; up to 4 views the two plain ones (0 and 3) are built, for 17 to
+// 32 views the default and the warp-per-ray one (fewer instantiations to build).
 template <int KMAX, typename MT, template <int, typename, typename> class F, typename T, typename... Args>
 void full_or_not(int K, Args... args) {
     if (K == KMAX) F<KMAX, MT, typename FullTile<T>::type>::run(args...);

@@ -130,6 +130,21 @@ cudaError_t launch_weight_map(const void *depth, int depth_dtype, void *map, int
                               float mu, float wconst, int window, cudaStream_t st, bool exact = false);
 cudaError_t launch_fuse(const FuseArgs &a, cudaStream_t st);
 
+// The variant (a tile of fuse_march.cuh) whose kernel a call runs.  Up to 8 views the default 0 is
+// the better of the two plain bundle shapes: 4 x 8 pixels (3) beats 8 x 4 unless the target is much
+// coarser than the views (us, 8 x 4 and 4 x 8: 8 x 1080p 236 and 227, 5 x 961x541 68 and 62,
+// 7 x 720p arc 122 and 109, 4 x 640x360 27 and 23, temporal 720p 146 and 144; 8 x 720p into 640x360
+// 71 and 75); for more views the two are level.  Not always, though (8 x 320x240, 128 samples: 49
+// and 57), so where 0 is 4 x 8, 1 is the plain 8 x 4: its own longer segments were at most 0.4 %
+// faster than that and up to 36 % slower, over 60 workloads of 5 to 8 views.  Up to 4 views there
+// is one choice, as every other number runs 0.
+inline int shaped_variant(int variant, int K, int64_t target_pixels, int64_t view_pixels) {
+    if (K > 8) return variant;
+    const int better = 2 * target_pixels >= view_pixels ? 3 : 0;
+    if (K <= 4 || variant == 0) return better;
+    return variant == 1 && better == 3 ? 0 : variant;
+}
+
 // Bundles of a target: the size of a launch.
 int bundle_count(int Wt, int Ht, int K, int variant);
 cudaError_t launch_fuse_batch(const FuseArgs *items, int n_items, int K, int map_dtype, int variant, cudaStream_t st);
