@@ -5,8 +5,8 @@ fastest on a given workload.
 Every variant computes the same fused depth bit for bit; only the time
 differs.  Each candidate is timed with CUDA events on the caller's stream
 after a warm-up, and the winner is cached in a JSON file keyed by the device
-(name, SM count) and a hash of the workload's shape, so a later process with
-the same workload reuses it without timing.
+(name, SM count), a hash of the library and a hash of the workload's shape, so
+a later process with the same library and workload reuses it without timing.
 """
 from __future__ import annotations
 
@@ -16,6 +16,8 @@ import os
 import threading
 
 import torch
+
+from . import gvs
 
 CACHE_PATH = os.environ.get("GVS_AUTOTUNE_CACHE",
                             os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build", "autotune.json"))
@@ -34,6 +36,12 @@ def variants_for(n_views: int, target_pixels: int = None, view_pixels: int = Non
             return tuple(v for v in VARIANTS if v != 3)
         return VARIANTS
     return (0, 6) if n_views > 16 else (0,)
+
+
+def library_key() -> str:
+    """Hash of the built library: a choice holds for the kernels it was timed with."""
+    with open(gvs.LIB_PATH, "rb") as f:
+        return hashlib.sha256(f.read()).hexdigest()[:16]
 
 
 def device_key() -> str:
@@ -86,7 +94,7 @@ def choose(shape: dict, make_runner, candidates=VARIANTS, use_cache: bool = True
     that enqueues one run of the workload with that variant."""
     if len(candidates) == 1:  # nothing to choose between
         return candidates[0], {}
-    key = device_key() + "|" + workload_key(**shape)
+    key = "|".join((device_key(), library_key(), workload_key(**shape)))
     if use_cache:
         hit = _load_cache().get(key)
         if hit is not None and hit.get("variant") in candidates:

@@ -1,5 +1,6 @@
-"""The fusion's variant numbers: every compiled bundle shape stays selectable and the autotuner
-times only distinct kernels.  No GPU."""
+"""The fusion's variant numbers: every compiled bundle shape stays selectable, the autotuner
+times only distinct kernels, and forgets its choices when the library is rebuilt.  No GPU."""
+import json
 import os
 import shutil
 import subprocess
@@ -54,3 +55,26 @@ def test_candidates_are_distinct_kernels(effective):
             if 5 <= k <= 16:
                 assert set(e) == {effective[v, k, t, p] for v in range(7)}
 
+
+def test_choice_is_forgotten_with_the_library(tmp_path, monkeypatch):
+    """A cached choice holds for the library it was timed with."""
+    from paper_2505_18932_gb300 import autotune, gvs
+    lib = tmp_path / "libgvs.so"
+    lib.write_bytes(b"one build")
+    monkeypatch.setattr(gvs, "LIB_PATH", str(lib))
+    monkeypatch.setattr(autotune, "CACHE_PATH", str(tmp_path / "autotune.json"))
+    monkeypatch.setattr(autotune, "device_key", lambda: "device")
+    monkeypatch.setattr(autotune, "time_ms", lambda fn: fn())
+    timed = []
+
+    def choose(ms):
+        def runner(v):
+            timed.append(v)
+            return lambda: ms[v]
+        return autotune.choose({"views": 8}, runner, candidates=(0, 1, 2))[0]
+
+    assert choose([3.0, 1.0, 2.0]) == 1 and timed == [0, 1, 2]
+    assert choose([1.0, 3.0, 2.0]) == 1 and timed == [0, 1, 2]       # from the cache
+    lib.write_bytes(b"another build")
+    assert choose([3.0, 2.0, 1.0]) == 2 and timed == [0, 1, 2] * 2   # timed again
+    assert len(json.load(open(autotune.CACHE_PATH))) == 2
