@@ -385,19 +385,20 @@ typedef struct {
 
 typedef struct gvs_fuse_batch gvs_fuse_batch;  /* opaque host object */
 
-/* Device table bytes for n_items items. */
+/* Device table bytes for n_items items: the least that is 256-byte aligned, as the items are
+ * kernel parameters. */
 GVS_API size_t gvs_fuse_batch_bytes(int32_t n_items);
 
 /* Validates the items (all with the same input views and params) and returns a
  * host handle that holds their descriptors.  `table` (device, caller-owned,
- * >= gvs_fuse_batch_bytes) is validated and reserved for the handle, but not
- * written.  The maps, outputs and table must outlive the handle. */
+ * >= gvs_fuse_batch_bytes, 256-byte aligned) is required but neither read nor written.
+ * No device work: it may be called during a stream capture.  The maps and outputs
+ * must outlive the handle. */
 GVS_API gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, const gvs_fuse_item *items,
                                          int32_t n_items, const gvs_fuse_params *params, void *table,
                                          size_t table_bytes, gvs_fuse_batch **out);
 
-/* Enqueues the batched fusion on `stream`.  Launches that share a table must
- * not overlap. */
+/* Enqueues the batched fusion on `stream`. */
 GVS_API gvs_status gvs_fuse_batch_launch(const gvs_fuse_batch *batch, void *stream);
 
 GVS_API void gvs_fuse_batch_destroy(gvs_fuse_batch *batch);

@@ -867,10 +867,7 @@ struct gvs_fuse_batch {
 
 extern "C" {
 
-size_t gvs_fuse_batch_bytes(int32_t n_items) {
-    if (n_items < 0) return 0;
-    return align_up((size_t)n_items * (sizeof(gvs::FuseArgs) + sizeof(int) * 2), 256) + 256;
-}
+size_t gvs_fuse_batch_bytes(int32_t n_items) { return n_items < 0 ? 0 : 256; }
 
 gvs_status gvs_fuse_batch_create(const gvs_camera *in_cams, int32_t n_views, const gvs_fuse_item *items,
                                  int32_t n_items, const gvs_fuse_params *params, void *table, size_t table_bytes,

@@ -852,7 +852,7 @@ class FuseBatch:
     """Batched fusion of many (map, target) items in shared launches (gvs_fuse_batch_*).
 
     items: list of (map_tensor, target_camera, fused_out [Ht, Wt] float32, crossing_out int16 or None).
-    Create outside any stream capture (it copies the item table); launch() may be captured."""
+    launch() may be captured."""
 
     def __init__(self, in_cams, items, num_samples, z_near, z_far, mu, normalize=False, map_half=False, variant=0):
         lib = load()
@@ -869,7 +869,7 @@ class FuseBatch:
         p = GvsFuseParams(int(num_samples), float(z_near), float(z_far), float(mu), 0.001, 7, int(bool(normalize)),
                           GVS_F32, GVS_F16 if map_half else GVS_F32, int(variant))
         dev = items[0][0].device
-        self.table = workspace(int(lib.gvs_fuse_batch_bytes(len(items))), dev)
+        self.table = workspace(int(lib.gvs_fuse_batch_bytes(len(items))), dev)  # asked for, not used
         h = ctypes.c_void_p()
         st = lib.gvs_fuse_batch_create(camera_array(in_cams), len(in_cams), arr, len(items), ctypes.byref(p),
                                        _ptr(self.table), self.table.numel(), ctypes.byref(h))
