@@ -68,6 +68,7 @@ extern "C" {
 #define GVS_MAX_SAMPLES 32767   /* samples per ray (crossing index is int16) */
 #define GVS_MAX_WINDOW 15       /* confidence window side (odd) */
 #define GVS_MAX_BATCH_ITEMS 1024 /* (frame, target) items of one batched fusion */
+#define GVS_BATCH_LAUNCH_ITEMS 14 /* of which so many share a launch */
 
 typedef enum {
     GVS_OK = 0,
@@ -371,7 +372,7 @@ GVS_API gvs_status gvs_soft_splat_backward(const gvs_camera *in_cams, const void
  * pattern; the paper has no counterpart, each item is Supplement A.1's fusion).  Each
  * item fuses the map of one frame (gvs_weight_map) into one target camera,
  * exactly as gvs_fuse_depth_from_map would; targets may differ in size.  A launch
- * takes up to 14 items, their arguments as kernel parameters and their blocks one
+ * takes up to GVS_BATCH_LAUNCH_ITEMS items, their arguments as kernel parameters and their blocks one
  * item after another in one grid (no block waits on another).  These are plain
  * kernel launches, so they can be captured in a CUDA graph.
  */

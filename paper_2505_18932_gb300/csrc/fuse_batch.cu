@@ -9,7 +9,7 @@ namespace {
 // arguments are the kernel's parameters: the march reads them from the constant bank, as
 // the single-item kernel does.  2 x 4 targets of 8 views: 1.16 ms as one persistent launch
 // with the arguments in shared memory, 1.10 as one launch per item, 1.04 so.
-constexpr int kBatchArgs = 14;
+constexpr int kBatchArgs = GVS_BATCH_LAUNCH_ITEMS;
 struct BatchArgs {
     FuseArgs item[kBatchArgs];
     unsigned first_block[kBatchArgs];

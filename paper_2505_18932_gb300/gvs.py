@@ -844,7 +844,7 @@ class SoftSplat(torch.autograd.Function):
         return gd, gc.to(in_color.dtype), None, None, None
 
 
-# Items of a batch that share a launch.
+# Items of a batch that share a launch (GVS_BATCH_LAUNCH_ITEMS).
 FUSE_BATCH_ITEMS = 14
 
 

@@ -1,5 +1,7 @@
 """Host side of the batched fusion: creation does no device work and holds no device memory."""
 import ctypes
+import os
+import re
 
 import pytest
 
@@ -40,3 +42,11 @@ def test_batch_table(lib, n_items):
     assert create(table=FAKE + 16) == 3
     assert create(n=0) == 1
     assert create(n=1025) == 1
+
+
+def test_items_of_a_launch():
+    """The binding counts launches with the library's own number of items."""
+    from paper_2505_18932_gb300 import gvs
+    h = open(os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "include", "gvs.h")).read()
+    n = int(re.search(r"#define GVS_BATCH_LAUNCH_ITEMS (\d+)", h).group(1))
+    assert gvs.FUSE_BATCH_ITEMS == n
