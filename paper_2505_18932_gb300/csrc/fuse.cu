@@ -377,7 +377,7 @@ struct FuseLaunch {
     static void run(const FuseArgs &a, cudaStream_t st) { launch_fuse_t<KMAX, MT, T, false>(a, st); }
 };
 
-// With the temporal input (Supplement A.2): the default tile only.
+// With the temporal input (Supplement A.2): the plain 8 x 4 and 4 x 8 tiles only.
 template <int KMAX, typename MT, typename T>
 struct FuseLaunchTemporal {
     static void run(const FuseArgs &a, cudaStream_t st) { launch_fuse_t<KMAX, MT, T, true>(a, st); }

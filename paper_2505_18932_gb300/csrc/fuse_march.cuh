@@ -261,16 +261,15 @@ __device__ __forceinline__ bool slab_view_free(const FuseArgs &a, const int2 *ta
 // A view whose sample lies behind its camera or off its image, or in front of
 // the surface by more than mu, enters with weight 0 (a predicated gather, no
 // branch): adding 0 * x leaves S and W as they were.
-// FULL: the call has exactly KMAX views (no per-view guard).  PLANES: address
-// view k's map through a.vb[k] (a constant-bank read for a __grid_constant__
-// FuseArgs); otherwise from a.dw (where the arguments sit in global memory).
+// FULL: the call has exactly KMAX views (no per-view guard).  View k's map plane is
+// a.vb[k], a constant-bank read of the kernel's parameters.
 //
 // With every view present, two views at a time (four of four) go through the same three
 // steps (pixels, gathers, sums) with one branch, for the rare pixel that needs the exact
 // decision: the group's gathers are in flight together.  8 x 1080p fusion kernel, in groups
 // of 1, 2, 4 and 8: 250, 236, 265 and 286 us (the larger ones spill); the sphere march
 // of 4 views 113, 105 and 101 us.
-template <int KMAX, typename MT, bool FULL = false, bool PLANES = true>
+template <int KMAX, typename MT, bool FULL = false>
 __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&ray)[KMAX], float zs, float &S,
                                                 float &Wsum) {
     constexpr int G = !FULL ? 1 : KMAX <= 4 ? KMAX : 2;
@@ -312,8 +311,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
                                       GVS_SITE_FUSE_MAP);
                 p[g] = make_float2(0.0f, 0.0f);
                 if (in[g]) {
-                    const MT *plane_k = PLANES ? reinterpret_cast<const MT *>(a.vb[k])
-                                               : reinterpret_cast<const MT *>(a.dw) + (size_t)k * plane;
+                    const MT *plane_k = reinterpret_cast<const MT *>(a.vb[k]);
                     p[g] = load_map(plane_k + (v[g] * a.W + u[g]));  // v W + u < 2^28
                 }
             }
@@ -331,7 +329,7 @@ __device__ __forceinline__ void evaluate_sample(const FuseArgs &a, const Ray (&r
 
 // Samples zs0 and zs1 at once (each exactly as evaluate_sample computes it): the
 // two samples' gathers of a view are independent, so a lane keeps both in flight.
-template <int KMAX, typename MT, bool FULL = false, bool PLANES = true>
+template <int KMAX, typename MT, bool FULL = false>
 __device__ __forceinline__ void evaluate_sample2(const FuseArgs &a, const Ray (&ray)[KMAX], float zs0, float zs1,
                                                  float &S0, float &W0, float &S1, float &W1) {
     const size_t plane = (size_t)a.W * a.H;
@@ -339,8 +337,7 @@ __device__ __forceinline__ void evaluate_sample2(const FuseArgs &a, const Ray (&
 #pragma unroll
     for (int k = 0; k < KMAX; ++k) {
         if (FULL || k < a.K) {
-            const MT *plane_k = PLANES ? reinterpret_cast<const MT *>(a.vb[k])
-                                       : reinterpret_cast<const MT *>(a.dw) + (size_t)k * plane;
+            const MT *plane_k = reinterpret_cast<const MT *>(a.vb[k]);
             float hz[2], pd[2], pw[2];
             bool in[2];
 #pragma unroll
@@ -379,9 +376,8 @@ __device__ __forceinline__ void evaluate_sample2(const FuseArgs &a, const Ray (&
 // evaluates sample s (all KMAX views unrolled, one 8-byte gather each) and
 // checks its own crossing.  The result equals the full uniform march.
 // TMP: the temporal input (previous output depth and weight) and the views'
-// weight at the crossing are compiled in only where they are used.  PLANES as
-// in evaluate_sample.
-template <int KMAX, typename MT, typename T, bool TMP = false, bool PLANES = true>
+// weight at the crossing are compiled in only where they are used.
+template <int KMAX, typename MT, typename T, bool TMP = false>
 __device__ __forceinline__ void march_rays(const FuseArgs &a, const int2 *tab, int bundle, int lane) {
     constexpr int BX = T::bx, BY = T::by, SKIP_LONG = T::llong, SKIP_SHORT = T::lshort;
     constexpr int NSEG = 32 / KMAX;
@@ -477,9 +473,9 @@ __device__ __forceinline__ void march_rays(const FuseArgs &a, const int2 *tab, i
         ze[0] = zs0;
         if (T::spt == 2 && nev == 2) {
             ze[1] = __fmaf_rn((float)(s + 1), a.dz, a.zn);
-            evaluate_sample2<KMAX, MT, T::full, PLANES>(a, ray, ze[0], ze[1], Se[0], We[0], Se[1], We[1]);
+            evaluate_sample2<KMAX, MT, T::full>(a, ray, ze[0], ze[1], Se[0], We[0], Se[1], We[1]);
         } else {
-            evaluate_sample<KMAX, MT, T::full, PLANES>(a, ray, zs0, Se[0], We[0]);
+            evaluate_sample<KMAX, MT, T::full>(a, ray, zs0, Se[0], We[0]);
         }
 #pragma unroll
         for (int e = 0; e < T::spt; ++e) {
@@ -530,7 +526,7 @@ __device__ __forceinline__ void march_rays(const FuseArgs &a, const int2 *tab, i
 // samples are then scanned in order, so the crossing, its index and its depth are
 // bit for bit those of march_rays (and of the full uniform march).  No temporal
 // input.
-template <int KMAX, typename MT, typename T, bool PLANES = true>
+template <int KMAX, typename MT, typename T>
 __device__ __forceinline__ void march_ray_warp(const FuseArgs &a, const int2 *tab, int pixel, int lane) {
     constexpr int NQ = 32 / KMAX;  // samples per step = segments per slab test
     constexpr unsigned SEGMASK = KMAX == 32 ? 0xffffffffu : ((1u << KMAX) - 1u);
@@ -544,8 +540,7 @@ __device__ __forceinline__ void march_ray_warp(const FuseArgs &a, const int2 *ta
     const SlabRays slab = slab_rays(a.xf[kk], i, i, j, j);
     const Ray ray = {slab.axlo, slab.aylo, slab.azlo};
     const float tb0 = slab.b0, tb1 = slab.b1, tb2 = slab.b2;
-    const MT *plane_k = PLANES ? reinterpret_cast<const MT *>(a.vb[kk])
-                               : reinterpret_cast<const MT *>(a.dw) + (size_t)kk * plane;
+    const MT *plane_k = reinterpret_cast<const MT *>(a.vb[kk]);
     float S_prev = 0.0f, W_prev = 0.0f, z_prev = 0.0f;
     bool have_prev = false;
     float out = 0.0f;
@@ -645,13 +640,13 @@ __device__ __forceinline__ void march_ray_warp(const FuseArgs &a, const int2 *ta
     }
 }
 
-template <int KMAX, typename MT, typename T, bool TMP = false, bool PLANES = true>
+template <int KMAX, typename MT, typename T, bool TMP = false>
 __device__ __forceinline__ void march_bundle(const FuseArgs &a, const int2 *tab, int bundle, int lane) {
     if constexpr (T::warp) {
         static_assert(!TMP, "the warp-per-ray march takes no temporal input");
-        march_ray_warp<KMAX, MT, T, PLANES>(a, tab, bundle, lane);
+        march_ray_warp<KMAX, MT, T>(a, tab, bundle, lane);
     } else {
-        march_rays<KMAX, MT, T, TMP, PLANES>(a, tab, bundle, lane);
+        march_rays<KMAX, MT, T, TMP>(a, tab, bundle, lane);
     }
 }
 

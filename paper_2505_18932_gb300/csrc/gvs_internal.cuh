@@ -145,7 +145,7 @@ inline int shaped_variant(int variant, int K, int64_t target_pixels, int64_t vie
     return variant == 1 && better == 3 ? 0 : variant;
 }
 
-// Bundles of a target: the size of a launch.
+// Bundles of a target by its variant's number, the measure of what a batch may hold.
 int bundle_count(int Wt, int Ht, int K, int variant);
 cudaError_t launch_fuse_batch(const FuseArgs *items, int n_items, int K, int map_dtype, int variant, cudaStream_t st);
 // acc: [K][H][W] float2 scratch; grad_depths written (not accumulated)

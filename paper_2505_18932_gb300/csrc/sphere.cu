@@ -50,7 +50,7 @@ __device__ __forceinline__ void sphere_sample(const FuseArgs &a, const Ray (&ray
 
 template <int KMAX, bool FULL>
 __device__ __forceinline__ void sphere_eval(const FuseArgs &a, const Ray (&ray)[KMAX], float z, float &S, float &W) {
-    if (FULL) evaluate_sample<KMAX, float2, true, true>(a, ray, z, S, W);
+    if (FULL) evaluate_sample<KMAX, float2, true>(a, ray, z, S, W);
     else sphere_sample<KMAX>(a, ray, z, S, W);
 }
 
