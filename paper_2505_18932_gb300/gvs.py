@@ -247,11 +247,14 @@ def _ptr(t):
     return t.data_ptr()
 
 
+# torch.cuda.current_stream().cuda_stream without building the Stream object, where torch has it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
-    if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream)
-    # torch.cuda.current_stream().cuda_stream without building the Stream object
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    if stream is None and _raw_stream is not None:
+        return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+    return ctypes.c_void_p((stream or torch.cuda.current_stream()).cuda_stream)
 
 
 def depth_dtype_of(t) -> int:
