@@ -13,9 +13,9 @@ namespace {
 //   dD/dd(q) += g_S omega [-1 < sdf < 1] / mu                 (the clamp)
 //   dD/dd(n) += g_S c domega(q)/dd(n)   for q's window entries n (the weight)
 // with g_S = dD/dS of that sample.  The weight's derivative is linear in
-// g_S c, so pass 1 (one thread per target pixel) accumulates, per sampled
+// g_S c, so pass 1 (a lane per target pixel and view) accumulates, per sampled
 // input pixel q, A(q) = sum g_S c and B(q) = sum g_S omega [...] / mu with one
-// float2 atomic per (sample, view); pass 2 (one thread per input pixel x)
+// float2 atomic per (sample, view); pass 2 (per input pixel x)
 // applies domega/dnu and the window:
 //   grad(x) = B(x) + P(x) sum_{entries n of x} 2 (d_x - d_n) [|d_x - d_n| < mu]
 //           + sum_{c whose window holds x, with multiplicity}
@@ -25,8 +25,8 @@ namespace {
 // -0.5 omega / nu = -0.5 omega^3 / (w^2 w_c^2), so a float2 map gives P(c)
 // from its stored omega without re-summing the window; for a half2 map (omega
 // rounded to half) nu is re-summed from the depths.  Nothing of size D x H x W
-// is stored; the bracketing samples are recomputed by the forward's own code,
-// so they are bit-identical to it.
+// is stored; the bracketing samples are recomputed with the forward's operations in
+// the forward's order (evaluate_sample), so S is the same bits.
 // ---------------------------------------------------------------------------
 
 // Pass 1.  Only target pixels with a crossing (and a non-zero upstream

@@ -80,7 +80,7 @@ constexpr int SKIP_COOL = 3;
 
 // Bundle shape and slab-test lengths of the march.  Every variant computes the
 // same result; they differ only in speed, and the autotuner picks one per
-// workload (gvs_fuse_params.variant).
+// workload (gvs_fuse_params.variant; shaped_variant gives the tile's number).
 //   bx x by : target pixels one warp marches together (bx * by = 32)
 //   llong   : samples per segment in the first slab test
 //   lshort  : samples per segment in the second test when the first fails

@@ -1,8 +1,8 @@
 // The paper's own raymarch for the image-based TSDF (Supplement A.1): from
 // z_near, advance by 0.8 s until s changes sign, then three bisection steps.
-// One thread per target ray; the per-view ray coefficients, the sample
-// evaluation and the nearest-pixel contract are those of the uniform march
-// (fuse_march.cuh).  Every operation that moves the march is an explicitly
+// One lane per target ray, in bundles of a warp that prove free space together; the
+// per-view ray coefficients, the sample evaluation, the nearest-pixel contract and the
+// slab test are those of the uniform march (fuse_march.cuh).  Every operation that moves the march is an explicitly
 // rounded FP32 operation and the weights come from the correctly rounded map,
 // so the trajectory, the evaluation count and the depth are reproducible bit
 // for bit on the host (see gvs_fuse_depth_sphere in gvs.h).
