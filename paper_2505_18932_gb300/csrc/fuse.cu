@@ -100,8 +100,9 @@ __global__ void __launch_bounds__(256, 8) weight_map_kernel(const DT *__restrict
     const int y0 = blockIdx.y * WM_TY - R;
     const int tid = threadIdx.y * WM_TX + threadIdx.x;
     if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-        // whole-view bounds, reduced into by depth_bounds with integer atomics on the float bits
-        reinterpret_cast<uint4 *>(map + L.off_g)[k] = make_uint4(0x7f800000u, 0xff800000u, ~0u, ~0u);
+        // whole-view bounds, reduced into by depth_bounds with unsigned atomics on the bits of positive
+        // floats: +inf and 0 (the bits of -inf would outdo every depth)
+        reinterpret_cast<uint4 *>(map + L.off_g)[k] = make_uint4(0x7f800000u, 0u, ~0u, ~0u);
     }
     const int tx = threadIdx.x, ty = threadIdx.y;
     {

@@ -35,7 +35,7 @@ cudaError_t launch_refine_soft(const uint32_t *rgba_t, const uint32_t *rgba_prev
 // any pixel box spanning at most two tiles per axis at level l is covered by
 // one O_l entry.  G holds the bounds of the whole view.  Sections are 256-byte
 // aligned.  A bound (DepthBound) is the smallest and largest valid depth of
-// its pixels (+inf / -inf where there is none) and a 64-bit mask of occupied
+// its pixels (+inf / -inf where there is none; 0 as G's largest) and a 64-bit mask of occupied
 // depth bins.  The bins are those of the FP32 bit pattern: bin(d) = bits(d)
 // >> 18 (exponent and the 5 leading mantissa bits: 32 bins per octave, 1.6 to
 // 3.1 % of the depth wide), monotone in d for d >= 0 and exact.  Bit b of a
