@@ -11,7 +11,7 @@
 // resolves 76 -> 68 us, the soft ones 156 -> 134).  At 1080p a slot is
 // 16.6 MB, which stays resident in the 126 MB L2 between scatter and resolve.
 //   clear   : fill every slot with ~0 (once per call)
-//   scatter : contract geometry of every source pixel (four per thread), atomicMin on
+//   scatter : contract geometry of every source pixel (one to four per thread), atomicMin on
 //             every covered target pixel
 //   resolve : every target pixel and view (two to eight per thread): decode the key,
 //             gather the winner's colour and write the outputs.
@@ -206,31 +206,31 @@ __device__ __forceinline__ void scatter_pixel(const SplatArgs &a, unsigned long 
         }
 }
 
-// SC_ROWS source pixels per thread, SC_BY rows apart (blocks cover 32 x 8 SC_ROWS pixels):
+// ROWS source pixels per thread, SC_BY rows apart (blocks cover 32 x 8 ROWS pixels):
 // their depth loads overlap and the view's coefficients (indexed constants, fetched by a
 // slow unit that was 60 % busy) are fetched once.  8 x 1080p: 112 us with one pixel and the
-// divisions, 107 without them, 89 and 85 with 2 and 4 pixels.
+// divisions, 107 without them, 89 and 85 with 2 and 4 pixels.  A thread takes its pixels'
+// footprints one after another, though; see launch_scatter.
 // DT: float or __half depth storage, widened to FP32.
 // REJECT: candidates in front of the fused surface (z < fused - mu_guide)
 // take no part in the depth test.
-constexpr int SC_ROWS = 4;
-template <typename DT, bool REJECT = false>
+template <typename DT, bool REJECT, int ROWS>
 __global__ void __launch_bounds__(SC_BX * SC_BY) splat_scatter(const SplatArgs a, int k0, unsigned tag) {
     const int u = blockIdx.x * SC_BX + threadIdx.x;
-    const int v0 = blockIdx.y * (SC_BY * SC_ROWS) + threadIdx.y;
+    const int v0 = blockIdx.y * (SC_BY * ROWS) + threadIdx.y;
     if (u >= a.W) return;
     const int kk = blockIdx.z;
     const int k = k0 + kk;
     const DT *depth = reinterpret_cast<const DT *>(a.depth) + (size_t)k * a.W * a.H;
     unsigned long long *slot = a.keys + (size_t)kk * a.Wt * a.Ht;
-    float d[SC_ROWS];
+    float d[ROWS];
 #pragma unroll
-    for (int n = 0; n < SC_ROWS; ++n) {
+    for (int n = 0; n < ROWS; ++n) {
         const int v = v0 + n * SC_BY;
         d[n] = v < a.H ? load_depth(depth + v * a.W + u) : 0.0f;  // 0: no pixel
     }
 #pragma unroll
-    for (int n = 0; n < SC_ROWS; ++n) {
+    for (int n = 0; n < ROWS; ++n) {
         const int v = v0 + n * SC_BY;
         Geo b;
         if (contract_either(a.v[k], u, v, d[n], a.Wt, a.Ht, a.footprint, a.max_hw, b))
@@ -243,8 +243,42 @@ inline unsigned group_tag(int group) { return 31u - (unsigned)group; }
 static_assert(GVS_MAX_VIEWS <= 32, "a group's tag has 5 bits");
 static_assert((int64_t)GVS_MAX_DIM * GVS_MAX_DIM <= (int64_t)1 << 28, "a source index has 28 bits");
 
-inline dim3 scatter_grid(int W, int H, int kn, int rows = 1) {
-    return dim3((unsigned)((W + SC_BX - 1) / SC_BX), (unsigned)((H + SC_BY * rows - 1) / (SC_BY * rows)), (unsigned)kn);
+inline dim3 scatter_grid(int W, int H, int kn) {
+    return dim3((unsigned)((W + SC_BX - 1) / SC_BX), (unsigned)((H + SC_BY - 1) / SC_BY), (unsigned)kn);
+}
+
+// The scatter of views k0 .. k0 + kn.  Four pixels per thread where the launch has many and a
+// footprint is usually 2 x 2 pixels, else one, so that the footprints' chains are short: (us, one
+// and four pixels) 2 views of 320x240 2.4 and 2.9, 1 of 640x360 3.0 and 3.4, 1 of 1280x720 7.8
+// and 7.1, 2 of 1080p 26.2 and 20.3; magnified twice, views 15 degrees aside: 2 of 320x240 3.9
+// and 9.5, 2 of 720p 19.4 and 24.8; magnified 1.5 times, 2 of 720p 13.7 and 12.1.  Large magnified
+// launches with rejection, whose loads of the fused depth overlap, take two: 8 of 720p, magnified
+// twice, 77 with one, 64 with two, 65 with four, and from aside 88, 77 and 94.
+constexpr int64_t SC_MANY = 800000;    // source pixels of a launch
+constexpr float SC_MAGNIFIED = 1.6f;   // ratio of the focal lengths
+template <typename DT, bool REJECT, int ROWS>
+void launch_scatter_rows(const SplatArgs &a, int k0, int kn, unsigned tag, cudaStream_t st) {
+    const dim3 grid((unsigned)((a.W + SC_BX - 1) / SC_BX), (unsigned)((a.H + SC_BY * ROWS - 1) / (SC_BY * ROWS)),
+                    (unsigned)kn);
+    splat_scatter<DT, REJECT, ROWS><<<grid, dim3(SC_BX, SC_BY), 0, st>>>(a, k0, tag);
+}
+template <typename DT, bool REJECT = false>
+void launch_scatter(const SplatArgs &a, int k0, int kn, unsigned tag, cudaStream_t st) {
+    const int64_t pixels = (int64_t)a.W * a.H * kn;
+    float ratio = 0.0f;
+    for (int k = k0; k < k0 + kn; ++k) ratio = fmaxf(ratio, a.v[k].f_ratio);
+    const bool magnified = !(ratio <= SC_MAGNIFIED);
+    if (pixels >= SC_MANY && !magnified) {
+        launch_scatter_rows<DT, REJECT, 4>(a, k0, kn, tag, st);
+        return;
+    }
+    if constexpr (REJECT) {
+        if (pixels >= 2 * SC_MANY) {
+            launch_scatter_rows<DT, REJECT, 2>(a, k0, kn, tag, st);
+            return;
+        }
+    }
+    launch_scatter_rows<DT, REJECT, 1>(a, k0, kn, tag, st);
 }
 
 // has: some candidate of this group (tag) reached the pixel; then w is the winner's source
@@ -876,7 +910,7 @@ void soft_groups(const SplatArgs &a, int K, cudaStream_t st) {
         const int kn = (K - k0) < slots ? (K - k0) : slots;
         const unsigned tag = group_tag(k0 / slots);
         const bool reset = k0 + kn < K;  // the accumulators serve another group
-        splat_scatter<DT><<<scatter_grid(a.W, a.H, kn, SC_ROWS), dim3(SC_BX, SC_BY), 0, st>>>(a, k0, tag);
+        launch_scatter<DT>(a, k0, kn, tag, st);
         soft_accum<DT, CT><<<scatter_grid(a.W, a.H, kn), dim3(SC_BX, SC_BY), 0, st>>>(a, k0);
         if (tma_soft_resolve_ok(a, HWt))
             soft_resolve_tma<<<dim3((unsigned)((HWt + ST_PX - 1) / ST_PX), (unsigned)kn), 256, 0, st>>>(a, k0, tag, reset);
@@ -905,14 +939,13 @@ cudaError_t launch_splat(const SplatArgs &a, int K, cudaStream_t st) {
     }
     for (int k0 = 0; k0 < K; k0 += slots) {
         const int kn = (K - k0) < slots ? (K - k0) : slots;
-        const dim3 g = scatter_grid(a.W, a.H, kn, SC_ROWS), b(SC_BX, SC_BY);
         const unsigned tag = group_tag(k0 / slots);
         if (a.depth_dtype == GVS_F16) {
-            if (a.guide_reject) splat_scatter<__half, true><<<g, b, 0, st>>>(a, k0, tag);
-            else splat_scatter<__half><<<g, b, 0, st>>>(a, k0, tag);
+            if (a.guide_reject) launch_scatter<__half, true>(a, k0, kn, tag, st);
+            else launch_scatter<__half>(a, k0, kn, tag, st);
         } else {
-            if (a.guide_reject) splat_scatter<float, true><<<g, b, 0, st>>>(a, k0, tag);
-            else splat_scatter<float><<<g, b, 0, st>>>(a, k0, tag);
+            if (a.guide_reject) launch_scatter<float, true>(a, k0, kn, tag, st);
+            else launch_scatter<float>(a, k0, kn, tag, st);
         }
         if (tma_resolve_ok(a, HWt))
             splat_resolve_tma<<<dim3((unsigned)((HWt + RT_PX - 1) / RT_PX), (unsigned)kn), 256, 0, st>>>(a, k0, tag);

@@ -64,3 +64,28 @@ def test_differentiable_splat(gvs, oracle_mod, target, slots):
     assert np.array_equal(out["depth"].view(np.uint32), ref["depth"].view(np.uint32))
     assert np.abs(out["color"] - ref["color"]).max() <= 1e-3
     np.testing.assert_allclose(out["wsum"], ref["wsum"], rtol=1e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1.55, 1.7])
+@pytest.mark.parametrize("reject", [False, True])
+@pytest.mark.parametrize("size", [(161, 157), (227, 222)])
+def test_scatter_of_many_pixels(gvs, oracle_mod, scale, reject, size):
+    """32 views in one launch (807,000 and 1,612,608 pixels: several per thread) and in a launch per view (one
+    per thread), to both sides of the magnification where that changes: as the oracle, bit for bit."""
+    from synth import configs
+    w = configs.tiny(*size, 32, 16)
+    t = configs.tiny(90, 64, 2, 16).targets[0]
+    t.fx = t.fy = w.inputs[0].fx * scale
+    rgb, d = w.render_inputs(0)
+    fused = np.full((64, 90), np.float32(np.median(d)), np.float32)
+    for dt in (torch.float32, torch.float16):
+        depth = to_dev(d).to(dt)
+        ref = oracle_mod.forward_splat(w.inputs, depth.float().cpu().numpy(), u32(rgb), t, mu_guide=0.25,
+                                       fused=fused.astype(np.float64), guide_reject=reject)
+        for slots in (32, 1):
+            out = gvs.forward_splat(w.inputs, depth, to_dev(u32(rgb)), t, fused=to_dev(fused), mu_guide=0.25,
+                                    guide_reject=reject, ws=gvs.workspace(slots * 90 * 64 * 8))
+            torch.cuda.synchronize()
+            assert np.array_equal(out["winner"].cpu().numpy(), ref["winner"])
+            assert np.array_equal(out["warped_depth"].cpu().numpy().view(np.uint32), ref["warped_depth"].view(np.uint32))
+        assert (ref["winner"] >= 0).any()
