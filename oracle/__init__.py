@@ -375,11 +375,12 @@ def blend(warped_rgba, alpha, warped_depth, fused, w, w_bg, i_bg):
     K, H, W = wr.shape
     out = np.empty((3, H, W), np.float64)
     L = ctypes.c_double(0.0)
-    rc = lib.orc_blend(K, W, H, _ptr(wr), _ptr(np.ascontiguousarray(alpha, np.uint8)),
-                       _ptr(np.ascontiguousarray(warped_depth, np.float32)),
-                       _ptr(np.ascontiguousarray(fused, np.float32)), _ptr(np.ascontiguousarray(w, np.float64)),
-                       _ptr(np.ascontiguousarray(w_bg, np.float64)), _ptr(np.ascontiguousarray(i_bg, np.float64)),
-                       _ptr(out), ctypes.addressof(L))
+    # named, so that what is converted lives through the call
+    al = np.ascontiguousarray(alpha, np.uint8)
+    wd, fz = np.ascontiguousarray(warped_depth, np.float32), np.ascontiguousarray(fused, np.float32)
+    wk, wb, ib = (np.ascontiguousarray(a, np.float64) for a in (w, w_bg, i_bg))
+    rc = lib.orc_blend(K, W, H, _ptr(wr), _ptr(al), _ptr(wd), _ptr(fz), _ptr(wk), _ptr(wb), _ptr(ib), _ptr(out),
+                       ctypes.addressof(L))
     if rc != 0:
         raise ValueError("orc_blend rejected its arguments")
     return out, L.value
